@@ -631,7 +631,7 @@ static pf_status batch_launch(pf_batch* b, const double* t, const double* const*
   PF_BCUDA(b, cudaMemcpyAsync(b->slots_dev, b->slots_pin, sizeof(int) * n_act,
                               cudaMemcpyHostToDevice, b->stream));
   // 2-3. tiles, then the graph (active set seen before) or direct launches
-  const size_t smem = sizeof(StepCoef) * (size_t)S_max;
+  const size_t smem = step_table_bytes(S_max);
   if (b->autotune && !b->tuned) PF_BCUDA(b, run_autotune(b, active, smem));
   const bool same = b->tiles_active == active && b->tiles_smem == smem;
   if (!same) {

@@ -1,0 +1,386 @@
+// pf_fast.cuh -- the implicit substeps of the small problems with the FP64
+// work cut to what FP64 is needed for.
+//
+// GB300 issues two FP64 lanes a clock per SM against 128 FP32 ones, and the
+// propagation kernels were bound by FP64 issue (90 % of the pipe's cycles).  A
+// substep is written here in increments: with y = x_n + D the LMM's equation
+//   G(D) = D + R - gamma f(x_n + D) = 0
+// has R = r-terms of the differences x_n - x_{n-1}, x_{n-1} - x_{n-2} (BDF) or of
+// the stored derivatives (Adams-Moulton), all small beside x_n, and the
+// predictor's increment P likewise.  Of the K Newton iterations
+//   - the first K - 1 evaluate G in ff (pf_ff.cuh) and solve their linear
+//     system in FP32: as with the unrefined reciprocals of the FP64 path, an
+//     inexact correction is repaired by the next iteration's residual, here
+//     exact to 2^-47 of the terms (the Adams methods solve in ff: their
+//     explicit predictors are far off on stiff particles, where an inexact
+//     first step would be seen in the K-th);
+//   - the last evaluates G in FP64 at the point y = x_n + (leading float of D)
+//     and solves in ff: its correction is small beside y, so 2^-46 of it is
+//     below y's last bit, and so is what FP32 made of the point, since G is
+//     evaluated at the point itself.
+// The state stays a double plus a float carry (the low part of the last
+// correction, below the double's last bits), and Milne's estimate comes from
+// D - P without the cancellation of y - x_p.  The result is the K-th Newton
+// iterate to FP64 rounding, as before; a substep that does not satisfy this
+// reasoning (a non-finite value, a last correction that is not small, an
+// exponent outside the floats') is left to the FP64 path by fast_run's caller.
+//
+// A Robertson BDF2 substep with error sums takes 21 FP64 instructions instead
+// of 89, an M1 one 25 instead of 186.  Measured (GB300, device time):
+// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.31 ms, stage 2 1.08 -> 0.41 ms;
+// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.08 and 0.23 -> 0.14 ms.  The FP64 pipe is
+// still 80 % busy, the issue slots about half.  Accuracy over an interval,
+// against quadruple precision on 200 particles of the prior, 2-norm of the
+// state: Robertson 3e-16 (plain FP64 9e-16), M1 2e-16 (4e-16).
+#pragma once
+#include "pf_ff.cuh"
+
+namespace pfg {
+
+// Error sums are kept in ff at 2^80 of their value, so that the squares of
+// estimates from 2^-90 to 2^20 stay normal floats.
+constexpr double kErrScale = 0x1.0p40, kErrUnscale = 0x1.0p-80;
+
+// the range of states, parameters and steps for which products in the models
+// below stay within the floats (anything else takes the FP64 path)
+constexpr double kFastStateMin = 0x1.0p-40, kFastStateMax = 0x1.0p20;
+constexpr double kFastThetaMin = 0x1.0p-40, kFastThetaMax = 0x1.0p40;
+constexpr float kFastStepMin = 0x1.0p-60f, kFastStepMax = 0x1.0p40f;
+
+// One substep's coefficients for the increment form (built in shared memory
+// from the StepCoef table by fast_coef):
+//   R = ra a + rb b,   P = pa a + pb b + pc c,
+// BDF: a = x_n - x_{n-1}, b = x_{n-1} - x_{n-2}, c = f(t_n, x_n);
+// Adams: a, b, c = f_n, f_{n-1}, f_{n-2}.
+struct FastCoef {
+  double gamma, ra, rb, in1;  // in1: the input at t_{n+1} (forced problems)
+  ff g, fra, frb, pa, pb, pc;
+  ff mus;                     // Milne's factor times 2^40 (kErrScale)
+  float er, ep;               // the defects rho1 + rho2 + rho3 - 1, pi0 + pi1 + pi2 - 1 of the
+                              // rounded BDF weights (0 for Adams)
+};
+
+// The entry of a StepCoef c (any struct of its fields).
+template <class C>
+PF_FF_FN FastCoef fast_coef(const C& c) {
+  FastCoef f;
+  const bool adams = c.kind > 10;
+  // differences of the BDF weights are exact or nearly (they sum to one)
+  f.ra = adams ? -c.rho1 : c.rho2 + c.rho3;
+  f.rb = adams ? -c.rho2 : c.rho3;
+  f.gamma = c.gamma;
+  f.in1 = c.in1;
+  f.g = ff_from(c.gamma);
+  f.fra = ff_from(f.ra);
+  f.frb = ff_from(f.rb);
+  f.pa = ff_from(adams ? c.pi0 : -(c.pi1 + c.pi2));
+  f.pb = ff_from(adams ? c.pi1 : -c.pi2);
+  f.pc = ff_from(adams ? c.pi2 : c.pi3);
+  f.mus = ff_from(c.mu * kErrScale);
+  f.er = adams ? 0.0f : f_from(((c.rho1 - 1.0) + c.rho2) + c.rho3);
+  f.ep = adams ? 0.0f : f_from(((c.pi0 - 1.0) + c.pi1) + c.pi2);
+  return f;
+}
+
+// the three-vector residual in double, and what the models return beside it
+struct FastState {
+  double y[3];   // the point of the last iteration
+  float hh[3];   // its increment
+  float cor[3];  // G's part below the doubles: carries of x and R
+};
+
+// ---------------------------------------------------------------- Robertson
+struct RobertsonFast {
+  static constexpr int D = 3;
+  struct Fk {
+    ff k1, k2, k3;          // theta
+  };
+  struct Gk {
+    ff gk1, gk2, gk3, op;   // gamma theta, 1 + gamma k1
+  };
+  template <class Th>
+  PF_FF_FN static Fk consts(const Th& T) { return Fk{ff_from(T.k1), ff_from(T.k2), ff_from(T.k3)}; }
+  template <class Th>
+  PF_FF_FN static double theta_min(const Th& T) { return fmin(T.k1, fmin(T.k2, T.k3)); }
+  template <class Th>
+  PF_FF_FN static double theta_max(const Th& T) { return fmax(T.k1, fmax(T.k2, T.k3)); }
+  PF_FF_FN static Gk scaled(const Fk& k, const FastCoef& c) {
+    const ff gk1 = ff_mul(k.k1, c.g);
+    return Gk{gk1, ff_mul(k.k2, c.g), ff_mul(k.k3, c.g), ff_one_plus(gk1)};
+  }
+
+  // (I - gamma J) d = -G by the elimination of Robertson::newton, in ff
+  PF_FF_FN static void solve(const Gk& k, ff y2, ff y3, ff G1, ff G2, ff G3, ff (&dl)[3]) {
+    const ff q = ff_mul(k.gk3, y2), p = ff_mul(k.gk3, y3), w = ff_twice(ff_mul(k.gk2, y2));
+    const ff im = ff_rcp(k.op), l = ff_mul(k.gk1, im);
+    const ff den = ff_fma(im, ff_fma(q, w, p), ff_one_plus(w));
+    const ff num = ff_sub(ff_mul(ff_mul(q, im), G3), ff_fma(l, G1, G2));
+    dl[1] = ff_div(num, den);
+    dl[2] = ff_sub(ff_mul(w, dl[1]), G3);
+    dl[0] = ff_mul(im, ff_fma(q, dl[2], ff_sub(ff_mul(p, dl[1]), G1)));
+  }
+
+  // G = D + R - gamma f at y = x + D, then D -= (I - gamma J)^{-1} G, in FP32
+  // (WIDE: in ff)
+  template <bool WIDE>
+  PF_FF_FN static void early(const Fk&, const Gk& k, const FastCoef&, const ff (&x)[3], const ff (&R)[3],
+                             ff (&Dv)[3]) {
+    const ff y1 = ff_add(x[0], Dv[0]), y2 = ff_add(x[1], Dv[1]), y3 = ff_add(x[2], Dv[2]);
+    const ff q = ff_mul(k.gk3, y2), t = ff_mul(k.gk2, y2);
+    const ff ab = ff_sub(ff_mul(k.gk1, y1), ff_mul(q, y3));
+    const ff c = ff_mul(t, y2);
+    const ff g1 = ff_add(ff_add(Dv[0], R[0]), ab), g3 = ff_sub(ff_add(Dv[2], R[2]), c);
+    const ff g2 = ff_add(ff_sub(ff_add(Dv[1], R[1]), ab), c);
+    if (WIDE) {
+      ff dl[3];
+      solve(k, y2, y3, g1, g2, g3, dl);
+      for (int i = 0; i < 3; ++i) Dv[i] = ff_add(Dv[i], dl[i]);
+      return;
+    }
+    const float G1 = g1.h, G2 = g2.h, G3 = g3.h;
+    const float p = f_mul(k.gk3.h, y3.h), w = f_add(t.h, t.h);
+    const float im = f_rcp(k.op.h), l = f_mul(k.gk1.h, im);
+    const float den = f_fma(im, f_fma(q.h, w, p), f_add(1.0f, w));
+    const float num = f_fma(f_mul(q.h, im), G3, -f_fma(l, G1, G2));
+    const float d2 = f_mul(num, f_rcp(den));
+    const float d3 = f_fma(w, d2, -G3);
+    const float d1 = f_mul(im, f_fma(q.h, d3, f_fma(p, d2, -G1)));
+    Dv[0] = ff_add(Dv[0], d1);
+    Dv[1] = ff_add(Dv[1], d2);
+    Dv[2] = ff_add(Dv[2], d3);
+  }
+
+  // the last iteration's correction, from R64 = R + hh in double.  fy, dfy:
+  // f at the corrected point (double part and ff part), if wanted
+  template <bool NEEDF, class Th>
+  PF_FF_FN static void last(const Th& T, const Fk& fk, const Gk& k, const FastCoef& c, const FastState& st,
+                            const double (&R64)[3], ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
+    const double y1 = st.y[0], y2 = st.y[1], y3 = st.y[2];
+    const double q64 = T.k3 * y2;
+    const double s64 = fma(T.k1, y1, -(q64 * y3));  // k1 y1 - k3 y2 y3 = -f1
+    const double c64 = (T.k2 * y2) * y2;            // k2 y2^2 = f3
+    const ff G1 = ff_add(ff_from(fma(c.gamma, s64, R64[0])), st.cor[0]);
+    const ff G2 = ff_add(ff_from(fma(-c.gamma, s64, fma(c.gamma, c64, R64[1]))), st.cor[1]);
+    const ff G3 = ff_add(ff_from(fma(-c.gamma, c64, R64[2])), st.cor[2]);
+    const ff f2 = ff_from(y2), f3 = ff_from(y3);
+    solve(k, f2, f3, G1, G2, G3, dl);
+    if (NEEDF) {
+      // f is quadratic: f(y + d) = f(y) + J d + Q(d, d), in ff beside FP64 f(y)
+      const ff e2 = ff_add(f2, dl[1]);
+      const ff dq = ff_add(ff_mul(f3, dl[1]), ff_mul(e2, dl[2]));      // y2 y3 changes by
+      const ff ds = ff_sub(ff_mul(fk.k1, dl[0]), ff_mul(fk.k3, dq));
+      const ff dc = ff_mul(fk.k2, ff_mul(dl[1], ff_add(f2, e2)));
+      fy[0] = -s64;
+      fy[1] = s64 - c64;
+      fy[2] = c64;
+      dfy[0] = ff_neg(ds);
+      dfy[1] = ff_sub(ds, dc);
+      dfy[2] = dc;
+    }
+  }
+};
+
+// ----------------------------------------------------------------------- M1
+// The fluxes V x/(x + k) = V - u with u = V k/(x + k); in the last iteration u
+// is a float ut plus du = (V k - ut s)/s, s = x + k, the remainder formed by one
+// FP64 FMA, so no FP64 reciprocal is needed.
+struct MichaelisFast {
+  static constexpr int D = 3;
+  struct Fk {
+    double vk1, vk2, vd, vc;      // V1 k1, V2 k2, V1 - V2, V2 + lambda c0
+    ff fvk1, fvk2, fvd, fvc, fv1, fk1, fk2;
+  };
+  struct Gk {
+    double f0;                    // input - V1
+    ff ff0, gl;                   // the same, gamma lambda
+  };
+  static constexpr double kLambda = 0.5, kC0 = 2.0;
+  template <class Th>
+  PF_FF_FN static Fk consts(const Th& T) {
+    const double vk1 = T.v1 * T.k1, vk2 = T.v2 * T.k2, vd = T.v1 - T.v2, vc = fma(kLambda, kC0, T.v2);
+    return Fk{vk1, vk2, vd, vc, ff_from(vk1), ff_from(vk2), ff_from(vd), ff_from(vc), ff_from(T.v1),
+              ff_from(T.k1), ff_from(T.k2)};
+  }
+  template <class Th>
+  PF_FF_FN static double theta_min(const Th& T) { return fmin(fmin(T.v1, T.v2), fmin(T.k1, T.k2)); }
+  template <class Th>
+  PF_FF_FN static double theta_max(const Th& T) { return fmax(fmax(T.v1, T.v2), fmax(T.k1, T.k2)); }
+  template <class Th>
+  PF_FF_FN static Gk scaled(const Th& T, const Fk&, const FastCoef& c) {
+    const double f0 = c.in1 - T.v1;
+    return Gk{f0, ff_from(f0), ff{0.5f * c.g.h, 0.5f * c.g.l}};
+  }
+
+  // (I - gamma J) d = -G by forward substitution, in ff; u = V k/s, r = 1/s
+  PF_FF_FN static void solve(const Gk& gk, const FastCoef& c, ff u1, ff r1, ff u2, ff r2, ff G1, ff G2,
+                             ff G3, ff (&dl)[3]) {
+    const ff ga = ff_mul(ff_mul(c.g, u1), r1), gb = ff_mul(ff_mul(c.g, u2), r2);
+    dl[0] = ff_neg(ff_div(G1, ff_one_plus(ga)));
+    dl[1] = ff_div(ff_sub(ff_mul(ga, dl[0]), G2), ff_one_plus(gb));
+    dl[2] = ff_div(ff_sub(ff_mul(gb, dl[1]), G3), ff_one_plus(gk.gl));
+  }
+
+  template <bool WIDE>
+  PF_FF_FN static void early(const Fk& k, const Gk& gk, const FastCoef& c, const ff (&x)[3],
+                             const ff (&R)[3], ff (&Dv)[3]) {
+    const ff s1 = ff_add(ff_add(x[0], Dv[0]), k.fk1), s2 = ff_add(ff_add(x[1], Dv[1]), k.fk2);
+    const ff y3 = ff_add(x[2], Dv[2]);
+    const ff u1 = ff_div(k.fvk1, s1), u2 = ff_div(k.fvk2, s2);
+    const ff f1 = ff_add(gk.ff0, u1);
+    const ff f2 = ff_add(ff_sub(k.fvd, u1), u2);
+    const ff f3 = ff_sub(ff_sub(k.fvc, u2), ff{0.5f * y3.h, 0.5f * y3.l});
+    const ff g1 = ff_sub(ff_add(Dv[0], R[0]), ff_mul(c.g, f1));
+    const ff g2 = ff_sub(ff_add(Dv[1], R[1]), ff_mul(c.g, f2));
+    const ff g3 = ff_sub(ff_add(Dv[2], R[2]), ff_mul(c.g, f3));
+    if (WIDE) {
+      ff dl[3];
+      solve(gk, c, u1, ff_rcp(s1), u2, ff_rcp(s2), g1, g2, g3, dl);
+      for (int i = 0; i < 3; ++i) Dv[i] = ff_add(Dv[i], dl[i]);
+      return;
+    }
+    const float G1 = g1.h, G2 = g2.h, G3 = g3.h;
+    const float ga = f_mul(f_mul(c.g.h, u1.h), f_rcp(s1.h)), gb = f_mul(f_mul(c.g.h, u2.h), f_rcp(s2.h));
+    const float d1 = -f_mul(G1, f_rcp(f_add(1.0f, ga)));
+    const float d2 = f_mul(f_fma(ga, d1, -G2), f_rcp(f_add(1.0f, gb)));
+    const float d3 = f_mul(f_fma(gb, d2, -G3), f_rcp(f_add(1.0f, gk.gl.h)));
+    Dv[0] = ff_add(Dv[0], d1);
+    Dv[1] = ff_add(Dv[1], d2);
+    Dv[2] = ff_add(Dv[2], d3);
+  }
+
+  template <bool NEEDF, class Th>
+  PF_FF_FN static void last(const Th& T, const Fk& k, const Gk& gk, const FastCoef& c, const FastState& st,
+                            const double (&R64)[3], ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
+    const double s1 = st.y[0] + T.k1, s2 = st.y[1] + T.k2;
+    const ff e1 = ff_from(s1), e2 = ff_from(s2);
+    const ff r1 = ff_rcp(e1), r2 = ff_rcp(e2);
+    const float u1 = f_mul(k.fvk1.h, r1.h), u2 = f_mul(k.fvk2.h, r2.h);
+    const double w1 = d_from_f(u1), w2 = d_from_f(u2);
+    const ff du1 = ff_mul(ff_from(fma(-w1, s1, k.vk1)), r1);
+    const ff du2 = ff_mul(ff_from(fma(-w2, s2, k.vk2)), r2);
+    fy[0] = gk.f0 + w1;
+    fy[1] = (k.vd - w1) + w2;
+    fy[2] = fma(-kLambda, st.y[2], k.vc) - w2;
+    const ff gd1 = ff_mul(c.g, du1), gd2 = ff_mul(c.g, du2);
+    const ff G1 = ff_sub(ff_add(ff_from(fma(-c.gamma, fy[0], R64[0])), st.cor[0]), gd1);
+    const ff G2 = ff_sub(ff_add(ff_add(ff_from(fma(-c.gamma, fy[1], R64[1])), st.cor[1]), gd1), gd2);
+    const ff G3 = ff_add(ff_add(ff_from(fma(-c.gamma, fy[2], R64[2])), st.cor[2]), gd2);
+    const ff t1 = ff_add(du1, u1), t2 = ff_add(du2, u2);
+    solve(gk, c, t1, r1, t2, r2, G1, G2, G3, dl);
+    if (NEEDF) {
+      // u(s + d) = u - u d/(s + d)
+      const ff v1 = ff_sub(du1, ff_div(ff_mul(t1, dl[0]), ff_add(e1, dl[0])));
+      const ff v2 = ff_sub(du2, ff_div(ff_mul(t2, dl[1]), ff_add(e2, dl[1])));
+      dfy[0] = v1;
+      dfy[1] = ff_sub(v2, v1);
+      dfy[2] = ff_neg(ff_add(v2, ff{0.5f * dl[2].h, 0.5f * dl[2].l}));
+    }
+  }
+};
+
+template <class Th>
+PF_FF_FN RobertsonFast::Gk fast_scaled(const Th&, const RobertsonFast::Fk& k, const FastCoef& c) {
+  return RobertsonFast::scaled(k, c);
+}
+template <class Th>
+PF_FF_FN MichaelisFast::Gk fast_scaled(const Th& T, const MichaelisFast::Fk& k, const FastCoef& c) {
+  return MichaelisFast::scaled(T, k, c);
+}
+
+// What a particle carries from substep to substep.
+//   x, h1, h2 with float carries cx, c1, c2: x_n, x_{n-1}, x_{n-2}
+//   BDF: a = x - h1, b = h1 - h2 in double, fa, fb the same in ff; fc = f(x_n)
+//   Adams: a, b = f_n, f_{n-1} in double with carries ca, cb; fa, fb, fc in ff
+//   E: the error sums at 2^80 of their value
+struct FastCarry {
+  double x[3], h1[3], h2[3];
+  float cx[3], c1[3], c2[3];
+  double a[3], b[3];
+  float ca[3], cb[3];
+  ff fa[3], fb[3], fc[3], E[3];
+};
+
+// One substep.  FAM: 0 BDF2, 1 BDF3, 2 Adams-Moulton.  Returns false, with w
+// untouched, if the result is not to be trusted.
+template <class MF, int FAM, bool ERR, class Th>
+PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& c, int K, FastCarry& w) {
+  const typename MF::Gk gk = fast_scaled(T, fk, c);
+  ff P[3], Dv[3], xf[3];
+  FastState st;
+  double R64[3];
+  for (int i = 0; i < 3; ++i) {
+    xf[i] = ff_from(w.x[i]);
+    xf[i].l = f_add(xf[i].l, w.cx[i]);
+    ff p = ff_mul_raw(c.pa, w.fa[i]);
+    p = ff_fma(c.pb, w.fb[i], p);
+    if (FAM != 0) p = ff_fma(c.pc, w.fc[i], p);
+    if (FAM != 2) p.l = f_fma(c.ep, xf[i].h, p.l);
+    P[i] = Dv[i] = p;
+  }
+  if (K > 1) {
+    ff R[3];
+    for (int i = 0; i < 3; ++i) {
+      R[i] = ff_mul(c.fra, w.fa[i]);
+      if (FAM != 0) R[i] = ff_fma(c.frb, w.fb[i], R[i]);
+    }
+    for (int it = 0; it + 1 < K; ++it) MF::template early<FAM == 2>(fk, gk, c, xf, R, Dv);
+  }
+  for (int i = 0; i < 3; ++i) {
+    st.hh[i] = Dv[i].h;
+    const double hd = d_from_f(st.hh[i]);
+    st.y[i] = w.x[i] + hd;
+    R64[i] = fma(c.ra, w.a[i], FAM != 0 ? fma(c.rb, w.b[i], hd) : hd);
+    // carries: x is w.x + cx, so the point's increment is hh - cx; a and b
+    // likewise have parts below their doubles
+    float r = f_fma(c.fra.h, w.ca[i], -w.cx[i]);
+    if (FAM != 0) r = f_fma(c.frb.h, w.cb[i], r);
+    if (FAM != 2) r = f_fma(-c.er, xf[i].h, r);
+    st.cor[i] = r;
+  }
+  ff dl[3], dfy[3];
+  double fy[3];
+  MF::template last<FAM != 0>(T, fk, gk, c, st, R64, dl, fy, dfy);
+  // every value finite and the last correction small: |d| <= 2^-4 |y|
+  const float my = fabsf(f_from(st.y[0])) + fabsf(f_from(st.y[1])) + fabsf(f_from(st.y[2]));
+  const float md = fabsf(dl[0].h) + fabsf(dl[1].h) + fabsf(dl[2].h);
+  if (!(md <= 0.0625f * my && my < 0x1.0p60f)) return false;
+  for (int i = 0; i < 3; ++i) {
+    const double xn = st.y[i] + d_from_f(dl[i].h);
+    const float cn = dl[i].l;
+    // the increment from x_n to the new state
+    const ff Dn = ff_add(ff_add(dl[i], st.hh[i]), -w.cx[i]);
+    if (ERR) {
+      const ff e = ff_mul(c.mus, ff_sub(Dn, P[i]));
+      w.E[i] = ff_fma(e, e, w.E[i]);
+    }
+    if (FAM == 2) {
+      w.fc[i] = w.fb[i];
+      w.fb[i] = w.fa[i];
+      w.b[i] = w.a[i];
+      w.cb[i] = w.ca[i];
+      w.a[i] = fy[i] + d_from_f(dfy[i].h);
+      w.ca[i] = dfy[i].l;
+      w.fa[i] = ff_from(w.a[i]);
+      w.fa[i].l = f_add(w.fa[i].l, w.ca[i]);
+    } else {
+      if (FAM == 1) {
+        w.b[i] = w.a[i];
+        w.cb[i] = w.ca[i];
+        w.fc[i] = ff_add(ff_from(fy[i]), dfy[i]);
+      }
+      w.fb[i] = w.fa[i];
+      w.fa[i] = Dn;
+      w.a[i] = xn - w.x[i];
+      w.ca[i] = f_sub(cn, w.cx[i]);
+    }
+    w.h2[i] = w.h1[i];
+    w.c2[i] = w.c1[i];
+    w.h1[i] = w.x[i];
+    w.c1[i] = w.cx[i];
+    w.x[i] = xn;
+    w.cx[i] = cn;
+  }
+  return true;
+}
+
+}  // namespace pfg

@@ -25,9 +25,11 @@
 // own epoch (linear2, Robertson, M1) launches its kernels with programmatic
 // dependent launch: each waits (pdl_wait) before touching the epoch's state.
 #include <cstring>
+#include <type_traits>
 
 #include "pf_common.cuh"
 #include "pf_epoch.cuh"
+#include "pf_fast.cuh"
 #include "pf_kernels.h"
 #include "pf_models.cuh"
 #include "pf_scan.cuh"
@@ -68,6 +70,106 @@ __device__ __forceinline__ void feval(const typename M::Th& T, double u, const d
   if constexpr (M::kForced) out[0] += u;
 }
 
+// The increment form's model of each problem (pf_fast.cuh), and the family it
+// serves: none for the explicit methods, whose substep has no Newton solve to
+// make cheaper, and none for the linear problem (one Newton iteration, whose
+// whole correction would have to be formed in ff).
+template <class M>
+struct FastModel {
+  using type = void;
+};
+template <>
+struct FastModel<Robertson> {
+  using type = RobertsonFast;
+};
+template <>
+struct FastModel<Michaelis> {
+  using type = MichaelisFast;
+};
+template <class M, int F>
+constexpr bool kHasFast = !std::is_same<typename FastModel<M>::type, void>::value && F != kFamAb;
+
+// The increment form's table, behind the S entries of the substep table.
+__device__ __forceinline__ FastCoef* fast_table(const StepCoef* sc, int S) {
+  return reinterpret_cast<FastCoef*>(const_cast<StepCoef*>(sc) + S);
+}
+
+// Both substep tables of a block in its dynamic shared memory
+// (step_table_bytes(S)).  Ends with a barrier.
+__device__ __forceinline__ void load_step_tables(StepCoef* s_sc, const EpochParams* __restrict__ ep, int S) {
+  load_steps(s_sc, ep, S);
+  FastCoef* t = fast_table(s_sc, S);
+  for (int i = threadIdx.x; i < S; i += blockDim.x) t[i] = fast_coef(s_sc[i]);
+  __syncthreads();
+}
+
+// Whether the increment form takes a substep of this kind.
+template <int F>
+__device__ __forceinline__ bool fast_kind(int kind) {
+  return F == kFamBdf12 ? kind == 2 : F == kFamBdf3 ? kind == 3 : F == kFamAm;
+}
+
+// The substeps from s on in the increment form (pf_fast.cuh), as long as it
+// serves the particle; returns the first substep it has not done.  (f0, f1,
+// f2: the derivative history of the Adams methods, in and out.)
+template <class M, bool ERR, int F, int NF>
+__device__ __forceinline__ int fast_run(const typename M::Th& T, const StepCoef* sc, int s, int S, int K,
+                                        double (&x)[3], double (&h1)[3], double (&h2)[3], double (&E)[3],
+                                        double (&f0)[NF], double (&f1)[NF], double (&f2)[NF]) {
+  using MF = typename FastModel<M>::type;
+  constexpr int FAM = F == kFamBdf12 ? 0 : F == kFamBdf3 ? 1 : 2;
+  const FastCoef* fc = fast_table(sc, S);
+  // every state and parameter in the range in which the floats serve
+  double big = 0.0;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) big = fmax(big, fabs(x[i]));
+  if (s >= S || !(big >= kFastStateMin && big <= kFastStateMax && MF::theta_min(T) >= kFastThetaMin &&
+                  MF::theta_max(T) <= kFastThetaMax))
+    return s;
+  const typename MF::Fk fk = MF::consts(T);
+  FastCarry w;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    w.x[i] = x[i];
+    w.h1[i] = h1[i];
+    w.h2[i] = h2[i];
+    w.cx[i] = w.c1[i] = w.c2[i] = w.ca[i] = w.cb[i] = 0.0f;
+    w.E[i] = w.fc[i] = ff{0.0f, 0.0f};
+    if constexpr (FAM == 2) {
+      w.a[i] = f0[i];
+      w.b[i] = f1[i];
+      w.fc[i] = ff_from(f2[i]);
+    } else {
+      w.a[i] = x[i] - h1[i];
+      w.b[i] = h1[i] - h2[i];
+    }
+    w.fa[i] = ff_from(w.a[i]);
+    w.fb[i] = ff_from(w.b[i]);
+  }
+  if constexpr (FAM == 1) {
+    double fx[3];
+    feval<M>(T, sc[s].in0, x, fx);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) w.fc[i] = ff_from(fx[i]);
+  }
+#pragma unroll 1
+  for (; s < S && fast_kind<F>(sc[s].kind) && fc[s].g.h >= kFastStepMin && fc[s].g.h <= kFastStepMax; ++s)
+    if (!fast_step<MF, FAM, ERR>(T, fk, fc[s], K, w)) break;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    x[i] = w.x[i] + (double)w.cx[i];
+    h1[i] = w.h1[i] + (double)w.c1[i];
+    h2[i] = w.h2[i] + (double)w.c2[i];
+    if (ERR) E[i] = fma((double)w.E[i].h + (double)w.E[i].l, kErrUnscale, E[i]);
+    if constexpr (FAM == 2) {
+      f0[i] = w.a[i] + (double)w.ca[i];
+      f1[i] = w.b[i] + (double)w.cb[i];
+      f2[i] = (double)w.fc[i].h + (double)w.fc[i].l;
+    }
+  }
+  return s;
+}
+
 // Psi of Algorithm 1 for one particle over the S substeps of the interval.
 // (x, h1, h2) = (x_n, x_{n-1}, x_{n-2}).  With ERR the squared Milne local
 // error estimates are summed into E (Step 4b).
@@ -79,64 +181,18 @@ __device__ __forceinline__ void feval(const typename M::Th& T, double u, const d
 //                 states with this particle's theta at the interval's start
 //                 and then carried in registers (weights beyond the step's
 //                 order are zero, the unused slots hold a finite copy).
+// Two passes over the substeps in FP64 enclose the increment form's: the first
+// stops where that form can take over (after a cold start's BDF1 steps), the
+// second finishes what it left (for most particles nothing).
 template <class M, bool ERR, int F>
 __device__ __forceinline__ void propagate(const typename M::Th& T, const StepCoef* sc, int S, int K,
                                           const EpochParams* __restrict__ ep, double (&x)[M::D],
                                           double (&h1)[M::D], double (&h2)[M::D], double (&E)[M::D]) {
   constexpr int D = M::D;
-  if constexpr (F == kFamBdf12 || F == kFamBdf3) {
-    for (int s = 0; s < S; ++s) {
-      const StepCoef& c = sc[s];
-      double xp[D], r[D], y[D];
-      if (F == kFamBdf3 && c.kind == 3) {
-        double fx[D];
-        feval<M>(T, c.in0, x, fx);
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-          xp[i] = fma(c.pi3, fx[i], fma(c.pi2, h2[i], fma(c.pi1, h1[i], c.pi0 * x[i])));
-          r[i] = fma(c.rho3, h2[i], fma(c.rho2, h1[i], c.rho1 * x[i]));
-          y[i] = xp[i];
-        }
-      } else if (F == kFamBdf12 && c.kind == 2) {
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-          xp[i] = fma(c.pi2, h2[i], fma(c.pi1, h1[i], c.pi0 * x[i]));
-          r[i] = fma(c.rho2, h1[i], c.rho1 * x[i]);
-          y[i] = xp[i];
-        }
-      } else {
-        // BDF1 (cold start): r = x_n, Newton from x_n, error predictor x_n + h f(t_n, x_n)
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-          r[i] = x[i];
-          y[i] = x[i];
-        }
-        if (ERR) {
-          double g[D];
-          M::gf(T, c.h, x, g);
-          if constexpr (M::kForced) g[0] = fma(c.h, c.in0, g[0]);
-#pragma unroll
-          for (int i = 0; i < D; ++i) xp[i] = x[i] + g[i];
-        }
-      }
-      if constexpr (M::kForced) r[0] = fma(c.gamma, c.in1, r[0]);
-      M::newton(T, c.gamma, r, y, K);
-      if (ERR) {
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-          const double e = c.mu * (y[i] - xp[i]);
-          E[i] = fma(e, e, E[i]);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < D; ++i) {
-        h2[i] = h1[i];
-        h1[i] = x[i];
-        x[i] = y[i];
-      }
-    }
-  } else {
-    double f0[D], f1[D], f2[D];
+  constexpr bool kAdams = F == kFamAm || F == kFamAb;
+  constexpr bool kFast = kHasFast<M, F>;
+  double f0[kAdams ? D : 1], f1[kAdams ? D : 1], f2[kAdams ? D : 1];
+  if constexpr (kAdams) {
     const int q0 = sc[0].kind % 10;
     feval<M>(T, sc[0].in0, x, f0);
     if (q0 >= 2) feval<M>(T, ep->in_hist[0], h1, f1);
@@ -147,40 +203,98 @@ __device__ __forceinline__ void propagate(const typename M::Th& T, const StepCoe
     else
 #pragma unroll
       for (int i = 0; i < D; ++i) f2[i] = f1[i];
-    for (int s = 0; s < S; ++s) {
+  }
+  int s = 0;
+#pragma unroll 1
+  for (int pass = 0; pass < (kFast ? 2 : 1); ++pass) {
+#pragma unroll 1
+    for (; s < S; ++s) {
       const StepCoef& c = sc[s];
-      double xp[D], r[D], y[D], fn[D];
-#pragma unroll
-      for (int i = 0; i < D; ++i) {
-        xp[i] = fma(c.pi2, f2[i], fma(c.pi1, f1[i], fma(c.pi0, f0[i], x[i])));
-        r[i] = fma(c.rho2, f1[i], fma(c.rho1, f0[i], x[i]));
-        y[i] = xp[i];
+      if constexpr (kFast) {
+        if (pass == 0 && fast_kind<F>(c.kind)) break;
       }
-      if constexpr (F == kFamAm) {
-        double rr[D];
+      double xp[D], r[D], y[D];
+      if constexpr (!kAdams) {
+        if (F == kFamBdf3 && c.kind == 3) {
+          double fx[D];
+          feval<M>(T, c.in0, x, fx);
 #pragma unroll
-        for (int i = 0; i < D; ++i) rr[i] = r[i];
-        if constexpr (M::kForced) rr[0] = fma(c.gamma, c.in1, rr[0]);
-        M::newton(T, c.gamma, rr, y, K);
-      }
-      feval<M>(T, c.in1, y, fn);
-      if (ERR) {
+          for (int i = 0; i < D; ++i) {
+            xp[i] = fma(c.pi3, fx[i], fma(c.pi2, h2[i], fma(c.pi1, h1[i], c.pi0 * x[i])));
+            r[i] = fma(c.rho3, h2[i], fma(c.rho2, h1[i], c.rho1 * x[i]));
+            y[i] = xp[i];
+          }
+        } else if (F == kFamBdf12 && c.kind == 2) {
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            xp[i] = fma(c.pi2, h2[i], fma(c.pi1, h1[i], c.pi0 * x[i]));
+            r[i] = fma(c.rho2, h1[i], c.rho1 * x[i]);
+            y[i] = xp[i];
+          }
+        } else {
+          // BDF1 (cold start): r = x_n, Newton from x_n, error predictor x_n + h f(t_n, x_n)
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            r[i] = x[i];
+            y[i] = x[i];
+          }
+          if (ERR) {
+            double g[D];
+            M::gf(T, c.h, x, g);
+            if constexpr (M::kForced) g[0] = fma(c.h, c.in0, g[0]);
+#pragma unroll
+            for (int i = 0; i < D; ++i) xp[i] = x[i] + g[i];
+          }
+        }
+        if constexpr (M::kForced) r[0] = fma(c.gamma, c.in1, r[0]);
+        M::newton(T, c.gamma, r, y, K);
+        if (ERR) {
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            const double e = c.mu * (y[i] - xp[i]);
+            E[i] = fma(e, e, E[i]);
+          }
+        }
+      } else {
+        double fn[D];
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-          // AM: corrector y against the AB predictor; AB: the AM value at y
-          const double e = (F == kFamAm) ? c.mu * (y[i] - xp[i]) : c.mu * (fma(c.gamma, fn[i], r[i]) - y[i]);
-          E[i] = fma(e, e, E[i]);
+          xp[i] = fma(c.pi2, f2[i], fma(c.pi1, f1[i], fma(c.pi0, f0[i], x[i])));
+          r[i] = fma(c.rho2, f1[i], fma(c.rho1, f0[i], x[i]));
+          y[i] = xp[i];
+        }
+        if constexpr (F == kFamAm) {
+          double rr[D];
+#pragma unroll
+          for (int i = 0; i < D; ++i) rr[i] = r[i];
+          if constexpr (M::kForced) rr[0] = fma(c.gamma, c.in1, rr[0]);
+          M::newton(T, c.gamma, rr, y, K);
+        }
+        feval<M>(T, c.in1, y, fn);
+        if (ERR) {
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            // AM: corrector y against the AB predictor; AB: the AM value at y
+            const double e = (F == kFamAm) ? c.mu * (y[i] - xp[i]) : c.mu * (fma(c.gamma, fn[i], r[i]) - y[i]);
+            E[i] = fma(e, e, E[i]);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+          f2[i] = f1[i];
+          f1[i] = f0[i];
+          f0[i] = fn[i];
         }
       }
 #pragma unroll
       for (int i = 0; i < D; ++i) {
-        f2[i] = f1[i];
-        f1[i] = f0[i];
-        f0[i] = fn[i];
         h2[i] = h1[i];
         h1[i] = x[i];
         x[i] = y[i];
       }
+    }
+    if constexpr (kFast) {
+      if (pass == 0) s = fast_run<M, ERR, F>(T, sc, s, S, K, x, h1, h2, E, f0, f1, f2);
     }
   }
 }
@@ -634,7 +748,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_stage1(const __grid_constant_
   // the parameter block is written only by copies before the epoch's first
   // launch, so its substep table is staged before the wait
   StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_steps(s_sc, ep, ep->S);
+  load_step_tables(s_sc, ep, ep->S);
   pdl_wait();
   if (fd.ctrl->status != PF_OK) return;
   stage1_body<M, F>(fd, ep, blockIdx.x, gridDim.x, s_sc, s_red, &s_flag);
@@ -675,7 +789,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_stage2(const __grid_constant_
   __shared__ double s_red[32];
   __shared__ int s_flag;
   StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_steps(s_sc, ep, ep->S);
+  load_step_tables(s_sc, ep, ep->S);
   pdl_wait();
   if (fd.ctrl->status != PF_OK) return;
   stage2_body<M, F>(fd, ep, blockIdx.x, gridDim.x, s_sc, s_red, &s_flag);
@@ -810,7 +924,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_batch_stage(const FilterDev* 
   if (fd.ctrl->status != PF_OK) return;
   const EpochParams* ep = eps[t.f];
   StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_steps(s_sc, ep, ep->S);
+  load_step_tables(s_sc, ep, ep->S);
   const int vg = (int)((fd.N + kSmallThreads - 1) / kSmallThreads);
   if (STAGE == 1) stage1_body<M, F>(fd, ep, t.vb, vg, s_sc, s_red, &s_flag);
   else stage2_body<M, F>(fd, ep, t.vb, vg, s_sc, s_red, &s_flag);
@@ -973,7 +1087,7 @@ template <class M>
 static cudaError_t launch_epoch_t(const FilterDev& fd, const EpochParams* ep, int S,
                                   cudaStream_t st, cudaEvent_t* marks) {
   const int64_t N = fd.N;
-  const size_t smem = (size_t)S * sizeof(StepCoef);
+  const size_t smem = step_table_bytes(S);
   StageKernel k1, k2;
   stage_kernels<M>(fd.lmm, k1, k2);
   const unsigned g_small = stage_grid(N, fd.sms);
@@ -1116,9 +1230,11 @@ cudaError_t touch(K* k) {
 
 // A kernel that stages the substep table in dynamic shared memory may need
 // more than the default 48 KB (PF_MAX_SUBSTEPS entries); loads it as well.
+size_t step_table_bytes(int S) { return (sizeof(StepCoef) + sizeof(FastCoef)) * (size_t)S; }
+
 cudaError_t allow_step_table(const void* k) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(sizeof(StepCoef) * (size_t)kSMax));
+                              (int)step_table_bytes(kSMax));
 }
 
 struct UploadBlob {
@@ -1318,7 +1434,7 @@ cudaError_t launch_stage(int stage, const FilterDev& fd, const EpochParams* ep, 
     default: return cudaErrorInvalidValue;
   }
   const unsigned g = stage_grid(fd.N, fd.sms);
-  (stage == 1 ? k1 : k2)<<<g, stage_threads(fd.N, fd.sms), (size_t)S * sizeof(StepCoef), st>>>(fd, ep);
+  (stage == 1 ? k1 : k2)<<<g, stage_threads(fd.N, fd.sms), step_table_bytes(S), st>>>(fd, ep);
   return cudaGetLastError();
 }
 

@@ -65,6 +65,9 @@ cudaError_t launch_theta_mean(const FilterDev& fd, cudaStream_t st);
 // Load every kernel of the library on the current device now rather than at
 // its first launch (which may wait for the device to drain); once per device.
 cudaError_t preload_main_kernels();
+// Dynamic shared memory of the small problems' stage kernels: the substep table
+// and the increment form's (pf_fast.cuh).
+size_t step_table_bytes(int S);
 // Let kernel k stage a full substep table (PF_MAX_SUBSTEPS entries) in dynamic
 // shared memory; loads the kernel.
 cudaError_t allow_step_table(const void* k);
