@@ -147,11 +147,9 @@ static size_t layout(pf_filter* f, char* base) {
   }
   f->fd.tsq = (double*)take(sizeof(double) * moment_blocks_max(sms));
   f->fd.part = (double*)take(sizeof(double) * moment_blocks_max(sms) * f->fd.nrec);
-  // model work arrays: the Brusselator's stage buffers; the 2D system's
-  // committed weights exp(lw - max lw), which the moments store for x-bar
-  f->fd.wk = (f->ode == PF_ODE_BRUSSELATOR1D) ? (double*)take(sizeof(double) * bruss_work_doubles(N))
-             : (f->ode == PF_ODE_ADVDIFF2D)   ? (double*)take(sizeof(double) * N)
-                                              : nullptr;
+  // the 2D system's committed weights exp(lw - max lw), which the moments store
+  // for x-bar
+  f->fd.wk = f->ode == PF_ODE_ADVDIFF2D ? (double*)take(sizeof(double) * N) : nullptr;
   f->fd.x0 = (const double*)take(sizeof(double) * d);
   f->fd.xbar = (double*)take(sizeof(double) * d);
   f->fd.ticket = (unsigned*)take(sizeof(unsigned) * 8);

@@ -134,7 +134,7 @@ struct FilterDev {
   double* pmax;     // per-tile running maximum of the earlier tiles' last c
   double* tsq;      // per-block sums of g^2 (first-stage ESS, moment_blocks_max(sms))
   double* part;     // moment partial records, moment_blocks_max(sms) * nrec
-  double* wk;       // model work arrays (Brusselator: r, predictor, error sums; 2D system: weights)
+  double* wk;       // 2D system: the weights x-bar needs
   unsigned* ticket; // 4 counters for the last-block pattern
   Ctrl* ctrl;
   int nrec;

@@ -76,7 +76,6 @@ cudaError_t preload_kernels();
 // Brusselator stage kernels (pf_bruss.cu): stage 1 or 2 of one epoch.
 cudaError_t launch_bruss_stage(int stage, const FilterDev& fd, const EpochParams* ep, int S,
                                cudaStream_t st);
-size_t bruss_work_doubles(int64_t N);
 // 2D advection-diffusion stage kernels (pf_advdiff.cu): one block per
 // particle, the whole state in shared memory.
 cudaError_t launch_ad_stage(int stage, const FilterDev& fd, const EpochParams* ep, int S,
