@@ -11,6 +11,8 @@
 #include <string>
 #include <vector>
 
+#include <unistd.h>
+
 #include "pf_filter.h"
 #include "pf_scan.cuh"
 
@@ -865,14 +867,49 @@ pf_status pf_reset(pf_filter* f) {
   return PF_OK;
 }
 
+// Write a byte of every page of an output buffer, so that the copy into it finds
+// the pages mapped: a copy into memory the caller has not touched yet faults
+// them in from the device's side, six times as slowly (25 MB: 4.2 ms against
+// 0.65 ms with the pages touched first).
+static void touch_pages(void* p, size_t bytes) {
+  static const size_t page = [] {
+    const long v = sysconf(_SC_PAGESIZE);
+    return v > 0 ? (size_t)v : (size_t)4096;
+  }();
+  volatile char* c = static_cast<volatile char*>(p);
+  for (size_t i = 0; i < bytes; i += page) c[i] = 0;
+  if (bytes) c[bytes - 1] = 0;
+}
+
 pf_status pf_get_ensemble(const pf_filter* cf, double* x, double* h1, double* h2, double* phi,
                           double* logw) {
   pf_filter* f = const_cast<pf_filter*>(cf);
   if (!f) return fail(nullptr, PF_ERR_INVALID_ARG, "filter is NULL");
   pf_status st = read_ctrl(f);
   if (st != PF_OK) return st;
-  const Ensemble& E = f->ctrl_host->cur ? f->fd.ens[1] : f->fd.ens[0];
+  const int cur = f->ctrl_host->cur;
+  const Ensemble& E = cur ? f->fd.ens[1] : f->fd.ens[0];
   const int64_t N = f->N;
+  if (!f->pool && f->shard_total == 0) {
+    // nothing is in flight (the stream was waited for), so the pending buffer
+    // is free for the reordered copy.  A session of a server may have an epoch
+    // in flight on its lane's stream, and a shard one in progress: those are
+    // reordered on the host.
+    const Ensemble& P = cur ? f->fd.ens[0] : f->fd.ens[1];
+    PF_CUDA(f, launch_rows(f->fd, cur, f->stream));
+    double* const dst[5] = {x, h1, h2, phi, logw};
+    const double* const src[5] = {P.x, P.h1, P.h2, P.phi, P.lw};
+    const int rows[5] = {f->d, f->d, f->d, f->p, 1};
+    for (int k = 0; k < 5; ++k) {
+      if (!dst[k]) continue;
+      const size_t bytes = sizeof(double) * (size_t)rows[k] * (size_t)N;
+      touch_pages(dst[k], bytes);
+      PF_CUDA(f, cudaMemcpyAsync(dst[k], src[k], bytes, cudaMemcpyDeviceToHost, f->stream));
+      f->d2h_bytes += (int64_t)bytes;
+    }
+    PF_CUDA(f, cudaStreamSynchronize(f->stream));
+    return PF_OK;
+  }
   std::vector<double> tmp;
   auto pull = [&](const double* src, int rows, double* dst) -> pf_status {
     if (!dst) return PF_OK;

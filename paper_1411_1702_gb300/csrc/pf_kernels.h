@@ -62,6 +62,9 @@ cudaError_t upload_small(void* dst, const void* src, size_t bytes, cudaStream_t 
 int moment_record_size(int ode);
 // Weighted theta-space mean of the committed ensemble into Ctrl::theta_mean.
 cudaError_t launch_theta_mean(const FilterDev& fd, cudaStream_t st);
+// The committed ensemble (buffer cur) in particle order into the pending buffer,
+// log weights normalised; only while no epoch is in progress.
+cudaError_t launch_rows(const FilterDev& fd, int cur, cudaStream_t st);
 // Load every kernel of the library on the current device now rather than at
 // its first launch (which may wait for the device to drain); once per device.
 cudaError_t preload_main_kernels();
