@@ -64,7 +64,7 @@ enum : uint32_t { kRngInit = 1, kRngTheta = 2, kRngInnov = 3, kRngResample = 4 }
 struct StepCoef {
   double h, gamma, rho1, rho2, pi0, pi1, pi2, mu;
   int kind;
-  int pad;
+  int ref;  // a substep of the interval whose gamma and rho1 this one's equal to 2^-36
   double rho3, pi3;
   double in0, in1;
 };

@@ -154,6 +154,15 @@ int build_substeps(int lmm, int spacing, double dt, int substeps, double q0, dou
       const int q = lmm % 10;
       adams_coefficients(lmm / 10, depth + 1 < q ? depth + 1 : q, h0, c);
     } else bdf1_coefficients(h0, c);
+    // the previous substep's reference serves if its weights differ by the
+    // rounding of the times only
+    c.ref = i;
+    if (i > 0) {
+      const StepCoef& r = tab[tab[i - 1].ref];
+      if (r.kind == c.kind && std::fabs(c.gamma - r.gamma) <= 0x1.0p-36 * r.gamma &&
+          std::fabs(c.rho1 - r.rho1) <= 0x1.0p-36 * std::fabs(r.rho1))
+        c.ref = tab[i - 1].ref;
+    }
     hprev2 = hprev1;
     hprev1 = h0;
     depth = depth < 2 ? depth + 1 : 2;

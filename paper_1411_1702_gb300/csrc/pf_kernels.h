@@ -83,8 +83,6 @@ cudaError_t launch_bruss_stage(int stage, const FilterDev& fd, const EpochParams
 // particle, the whole state in shared memory.
 cudaError_t launch_ad_stage(int stage, const FilterDev& fd, const EpochParams* ep, int S,
                             cudaStream_t st);
-size_t ad_stage_smem(int d, int S, int stage);
-int ad_threads(int nt);
 cudaError_t preload_ad_kernels();
 int max_grid_blocks(int64_t N, int sms);
 int scan_tiles(int64_t N, int sms);
