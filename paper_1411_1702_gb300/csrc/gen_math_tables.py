@@ -7,6 +7,7 @@ cosine of pf_math.cuh, each entry the double nearest the exact value
   kPfLogInvF[j] = 1 / F_j,  F_j = 1 + j/128, j = 0..128
   kPfLogF[j] = log F_j,  kPfLogF[129 + j] = log(F_j / 2)
   kPfSinPi64[j] = sin(pi j / 64),  kPfCosPi64[j] = cos(pi j / 64),  j = 0..128
+  kPfExp2[j] = 2^(j/128) 2^61, j = 0..127, the integer nearest
 """
 from __future__ import annotations
 
@@ -47,15 +48,19 @@ def main():
         sin_t[j] = 0.0
     for j in (N_TRIG // 2, 3 * N_TRIG // 2):
         cos_t[j] = 0.0
+    exp2 = [int(mpmath.nint(mpmath.mpf(2) ** (mpmath.mpf(j) / 128) * 2 ** 61)) for j in range(128)]
+    rows = [", ".join(f"{v}LL" for v in exp2[i:i + 4]) for i in range(0, 128, 4)]
+    etab = "PF_TABLE int64_t kPfExp2[128] = {\n" + "\n".join("    " + r + "," for r in rows) + "\n};\n"
     text = (
         "// pf_mathtab.h -- tables of pf_math.cuh, written by gen_math_tables.py (do not edit):\n"
-        "// each entry is the double nearest the exact value.\n"
-        "#pragma once\n\n"
+        "// each entry is the double (or integer) nearest the exact value.\n"
+        "#pragma once\n#include <stdint.h>\n\n"
         "#ifdef __CUDACC__\n#define PF_TABLE __device__ const\n#else\n#define PF_TABLE static const\n#endif\n\n"
         "// 1 / F_j, and log F_j then log(F_j / 2), F_j = 1 + j/128\n"
         + table("kPfLogInvF", inv_f) + "\n" + table("kPfLogF", log_f) + "\n"
         "// sin(pi j/64) and cos(pi j/64)\n"
-        + table("kPfSinPi64", sin_t) + "\n" + table("kPfCosPi64", cos_t)
+        + table("kPfSinPi64", sin_t) + "\n" + table("kPfCosPi64", cos_t) + "\n"
+        "// 2^(j/128) 2^61\n" + etab
     )
     with open(OUT, "w") as f:
         f.write(text)

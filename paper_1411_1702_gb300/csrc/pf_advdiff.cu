@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
         }
       }
     }
-    for (int i = 0; i < 5; ++i) s_th[q][i] = (fd.transform == PF_TRANSFORM_LOG) ? exp(ph[i]) : ph[i];
+    for (int i = 0; i < 5; ++i) s_th[q][i] = (fd.transform == PF_TRANSFORM_LOG) ? pfm::exp_fixed(ph[i]) : ph[i];
   }
   ad_tables(L, sm, S);
   if (tid < 6 * PB) s_top[tid / (2 * PB)][tid % (2 * PB)] = 0u;
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
         const int i = 2 * b + h;
         if (i >= d) break;
         const double E = fma(value_of(reinterpret_cast<ff*>(R + L.F[2])[i]), kErrUnscale, R[L.F[1] + i]);
-        R[L.F[2] + i] = sqrt(fd.kappa * E) * (h == 0 ? z0 : z1);
+        R[L.F[2] + i] = pfm::sqrt_fixed(fd.kappa * E) * (h == 0 ? z0 : z1);
       }
     }
     __syncthreads();

@@ -541,7 +541,7 @@ __device__ __forceinline__ void bstage2_body(const FilterDev& fd, const EpochPar
       const int k = 2 * b + h;
       const int64_t o = (int64_t)(4 * g + k) * N + n;
       const double E = ((double)w.E[k].h + (double)w.E[k].l) * kErrUnscale;
-      const double v = sqrt(fd.kappa * E) * (h == 0 ? z0 : z1);
+      const double v = pfm::sqrt_fixed(fd.kappa * E) * (h == 0 ? z0 : z1);
       const double xk = w.x[k] + (double)w.cx[k];
       const double h1 = xk - (w.a[k] + (double)w.ca[k]);
       const double h2 = h1 - ((double)w.fb[k].h + (double)w.fb[k].l);

@@ -14,7 +14,7 @@ __device__ __forceinline__ Ensemble pending(const FilterDev& fd, int cur) {
 template <int P>
 __device__ __forceinline__ void to_theta(const FilterDev& fd, const double (&ph)[P], double (&th)[P]) {
 #pragma unroll
-  for (int i = 0; i < P; ++i) th[i] = (fd.transform == PF_TRANSFORM_LOG) ? exp(ph[i]) : ph[i];
+  for (int i = 0; i < P; ++i) th[i] = (fd.transform == PF_TRANSFORM_LOG) ? pfm::exp_fixed(ph[i]) : ph[i];
 }
 
 __device__ __forceinline__ void load_steps(StepCoef* s_sc, const EpochParams* __restrict__ ep, int S) {

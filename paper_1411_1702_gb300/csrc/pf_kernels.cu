@@ -475,7 +475,7 @@ __device__ __forceinline__ void stage2_body(const FilterDev& fd, const EpochPara
       for (int h = 0; h < 2; ++h) {
         const int i = 2 * b + h;
         if (i < D) {
-          const double v = sqrt(fd.kappa * Eacc[i]) * (h == 0 ? z0 : z1);
+          const double v = pfm::sqrt_fixed(fd.kappa * Eacc[i]) * (h == 0 ? z0 : z1);
           x[i] += v;
           h1[i] += v;
           h2[i] += v;
@@ -601,7 +601,7 @@ __device__ __forceinline__ void moments_body(const FilterDev& fd, int is_init, i
       if constexpr (D == 0) fd.wk[n] = 0.0;
       continue;
     }
-    const double e = exp(lw - M);
+    const double e = pfm::exp_fixed(lw - M);
     if constexpr (D == 0) fd.wk[n] = e;  // the weights x-bar needs (k_xbar)
     acc[Lay::kS0] += e;
     acc[Lay::kW2] = fma(e, e, acc[Lay::kW2]);
@@ -823,11 +823,11 @@ __global__ void __launch_bounds__(kMomentThreads) k_theta_mean(const __grid_cons
   for (int64_t n = threadIdx.x; n < N; n += blockDim.x) {
     const double lw = E.lw[n];
     if (is_neg_inf(lw)) continue;
-    const double w = exp(lw - lW);
+    const double w = pfm::exp_fixed(lw - lW);
 #pragma unroll
     for (int i = 0; i < P; ++i) {
       const double ph = E.phi[i * N + n];
-      acc[i] = fma(w, (fd.transform == PF_TRANSFORM_LOG) ? exp(ph) : ph, acc[i]);
+      acc[i] = fma(w, (fd.transform == PF_TRANSFORM_LOG) ? pfm::exp_fixed(ph) : ph, acc[i]);
     }
   }
   block_sum_vec<P>(acc, s_part, s_tot);

@@ -124,7 +124,7 @@ __host__ __device__ constexpr int scan_tile_count(int64_t N, int sms) {
 // finite or -inf).  A zero weight stays 0 whatever M is, so all-zero weights
 // give c = 0.
 __device__ __forceinline__ double scan_weight(double lg, double M) {
-  return finite_bits(lg) ? exp(lg - M) : 0.0;
+  return finite_bits(lg) ? pfm::exp_fixed(lg - M) : 0.0;
 }
 
 // The maximum of two doubles >= +0 (every partial sum here is): their order is

@@ -1,7 +1,7 @@
 // math_probe.cu -- the device side of the test of pf_math.cuh, in the probe
 // library (libpf_fp64_probe.so, outside the sampler's C ABI): evaluates the
-// table-driven logarithm and sine/cosine on the GPU for given inputs, so that
-// a test can compare them bit for bit with a host build of the same header.
+// table-driven logarithm and sine/cosine, and the fixed-point exp and sqrt, on the
+// GPU for given inputs, so that a test can compare them bit for bit with a host build of the same header.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -20,7 +20,25 @@ __global__ void k_math(const double* __restrict__ x, const uint64_t* __restrict_
   c[i] = b;
 }
 
+__global__ void k_fixed(const double* __restrict__ x, int64_t n, double* __restrict__ e, double* __restrict__ r) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  e[i] = pfm::exp_fixed(x[i]);
+  r[i] = pfm::sqrt_fixed(x[i]);
+}
+
 }  // namespace
+
+// exp x and sqrt x of x[n] into e and r (device memory, checked by the caller).
+// Synchronous.  Returns as pf_probe_math.
+extern "C" int pf_probe_fixed(const double* x, int64_t n, double* e, double* r) {
+  if (!x || !e || !r || n < 0 || n >= ((int64_t)1 << 31)) return -1;
+  if (n == 0) return 0;
+  k_fixed<<<(unsigned)((n + 255) / 256), 256>>>(x, n, e, r);
+  cudaError_t st = cudaGetLastError();
+  if (st == cudaSuccess) st = cudaDeviceSynchronize();
+  return (int)st;
+}
 
 // x[n]: positive normal doubles; k[n]: integers below 2^53 (all device
 // memory, checked by the caller).  Writes log x, sin(pi k 2^-52) and
