@@ -39,6 +39,16 @@ namespace pfg {
 constexpr int kSmallThreads = 128;
 constexpr int kInitThreads = 256;
 
+// Blocks of 128 stage threads an SM must hold, which bounds the registers: 128
+// for Robertson, 168 for M1 (and the linear problem uses fewer than either).
+// More warps hide the waits on FP64 results.  Unbounded, Robertson's stage 2 took 159
+// registers and M1's 188, whose 10 resident warps an SM left M1's 10.3 warps an SM at N
+// = 50000 with a second wave: M1 stage 2 0.129 -> 0.088 ms, AM3's 0.152 -> 0.101;
+// Robertson stage 2 0.373 -> 0.347 ms at N = 131072.  168 for Robertson slowed its
+// stage 1 by 17 % and 128 for M1 both of its stages by 4 %.
+template <class M>
+constexpr int kStageBlocks = M::ODE == PF_ODE_MICHAELIS3 ? 3 : 4;
+
 // Gaussian log-likelihood of the observed components, without the constant
 // terms (they cancel in every normalisation of Steps 3a and 5).
 template <int D>
@@ -740,7 +750,7 @@ __global__ void __launch_bounds__(kInitThreads) k_init(const __grid_constant__ F
 }
 
 template <class M, int F>
-__global__ void __launch_bounds__(kSmallThreads) k_stage1(const __grid_constant__ FilterDev fd,
+__global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_stage1(const __grid_constant__ FilterDev fd,
                                                           const EpochParams* __restrict__ ep) {
   extern __shared__ double s_dyn[];
   __shared__ double s_red[32];
@@ -783,7 +793,7 @@ __global__ void __launch_bounds__(kResampleThreads, 4) k_resample(const __grid_c
 }
 
 template <class M, int F>
-__global__ void __launch_bounds__(kSmallThreads) k_stage2(const __grid_constant__ FilterDev fd,
+__global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_stage2(const __grid_constant__ FilterDev fd,
                                                           const EpochParams* __restrict__ ep) {
   extern __shared__ double s_dyn[];
   __shared__ double s_red[32];
@@ -957,7 +967,7 @@ __global__ void __launch_bounds__(kInitThreads) k_batch_init(const FilterDev* __
 }
 
 template <class M, int STAGE, int F>
-__global__ void __launch_bounds__(kSmallThreads) k_batch_stage(const FilterDev* __restrict__ fds,
+__global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_batch_stage(const FilterDev* __restrict__ fds,
                                                              const EpochParams* const* __restrict__ eps,
                                                              const BatchTile* __restrict__ tiles) {
   extern __shared__ double s_dyn[];
