@@ -25,13 +25,14 @@
 // reasoning (a non-finite value, a last correction that is not small, an
 // exponent outside the floats') is left to the FP64 path by fast_run's caller.
 //
-// A Robertson BDF2 substep with error sums takes 21 FP64 instructions instead
-// of 89, an M1 one 25 instead of 186.  Measured (GB300, device time):
-// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.31 ms, stage 2 1.08 -> 0.41 ms;
-// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.08 and 0.23 -> 0.14 ms.  The FP64 pipe is
-// still 80 % busy, the issue slots about half.  Accuracy over an interval,
-// against quadruple precision on 200 particles of the prior, 2-norm of the
-// state: Robertson 3e-16 (plain FP64 9e-16), M1 2e-16 (4e-16).
+// A Robertson BDF2 substep with error sums takes 18 FP64 instructions instead
+// of 89, an M1 one 22 instead of 186.  Measured (GB300, device time):
+// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.275 ms, stage 2 1.08 -> 0.319 ms;
+// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.072 and 0.23 -> 0.085 ms (the exponentials and
+// roots of pf_math.cuh and the register bounds included).  The FP64 pipe is still
+// about 80 % busy, the issue slots 55 %.  Accuracy over an interval, against
+// quadruple precision on 200 particles of the prior, 2-norm of the state:
+// Robertson 2e-16 (plain FP64 9e-16), M1 2e-16 (4e-16).
 #pragma once
 #include "pf_ff.cuh"
 
@@ -82,11 +83,11 @@ PF_FF_FN FastCoef fast_coef(const C& c) {
   return f;
 }
 
-// the three-vector residual in double, and what the models return beside it
+// the point of the last iteration, x_n + hh, and D + R of its residual: the leading
+// part in double, the rest in ff
 struct FastState {
-  double y[3];   // the point of the last iteration
-  float hh[3];   // its increment
-  float cor[3];  // G's part below the doubles: carries of x and R
+  double y[3], R64[3];
+  ff cor[3];
 };
 
 // ---------------------------------------------------------------- Robertson
@@ -150,18 +151,18 @@ struct RobertsonFast {
     Dv[2] = ff_add(Dv[2], d3);
   }
 
-  // the last iteration's correction, from R64 = R + hh in double.  fy, dfy:
-  // f at the corrected point (double part and ff part), if wanted
+  // the last iteration's correction.  fy, dfy: f at the corrected point (double
+  // part and ff part), if wanted
   template <bool NEEDF, class Th>
   PF_FF_FN static void last(const Th& T, const Fk& fk, const Gk& k, const FastCoef& c, const FastState& st,
-                            const double (&R64)[3], ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
+                            ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
     const double y1 = st.y[0], y2 = st.y[1], y3 = st.y[2];
     const double q64 = T.k3 * y2;
     const double s64 = fma(T.k1, y1, -(q64 * y3));  // k1 y1 - k3 y2 y3 = -f1
     const double c64 = (T.k2 * y2) * y2;            // k2 y2^2 = f3
-    const ff G1 = ff_add(ff_from(fma(c.gamma, s64, R64[0])), st.cor[0]);
-    const ff G2 = ff_add(ff_from(fma(-c.gamma, s64, fma(c.gamma, c64, R64[1]))), st.cor[1]);
-    const ff G3 = ff_add(ff_from(fma(-c.gamma, c64, R64[2])), st.cor[2]);
+    const ff G1 = ff_add(ff_from(fma(c.gamma, s64, st.R64[0])), st.cor[0]);
+    const ff G2 = ff_add(ff_from(fma(-c.gamma, s64, fma(c.gamma, c64, st.R64[1]))), st.cor[1]);
+    const ff G3 = ff_add(ff_from(fma(-c.gamma, c64, st.R64[2])), st.cor[2]);
     const ff f2 = ff_from(y2), f3 = ff_from(y3);
     solve(k, f2, f3, G1, G2, G3, dl);
     if (NEEDF) {
@@ -250,7 +251,7 @@ struct MichaelisFast {
 
   template <bool NEEDF, class Th>
   PF_FF_FN static void last(const Th& T, const Fk& k, const Gk& gk, const FastCoef& c, const FastState& st,
-                            const double (&R64)[3], ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
+                            ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
     const double s1 = st.y[0] + T.k1, s2 = st.y[1] + T.k2;
     const ff e1 = ff_from(s1), e2 = ff_from(s2);
     const ff r1 = ff_rcp(e1), r2 = ff_rcp(e2);
@@ -262,9 +263,9 @@ struct MichaelisFast {
     fy[1] = (k.vd - w1) + w2;
     fy[2] = fma(-kLambda, st.y[2], k.vc) - w2;
     const ff gd1 = ff_mul(c.g, du1), gd2 = ff_mul(c.g, du2);
-    const ff G1 = ff_sub(ff_add(ff_from(fma(-c.gamma, fy[0], R64[0])), st.cor[0]), gd1);
-    const ff G2 = ff_sub(ff_add(ff_add(ff_from(fma(-c.gamma, fy[1], R64[1])), st.cor[1]), gd1), gd2);
-    const ff G3 = ff_add(ff_add(ff_from(fma(-c.gamma, fy[2], R64[2])), st.cor[2]), gd2);
+    const ff G1 = ff_sub(ff_add(ff_from(fma(-c.gamma, fy[0], st.R64[0])), st.cor[0]), gd1);
+    const ff G2 = ff_sub(ff_add(ff_add(ff_from(fma(-c.gamma, fy[1], st.R64[1])), st.cor[1]), gd1), gd2);
+    const ff G3 = ff_add(ff_add(ff_from(fma(-c.gamma, fy[2], st.R64[2])), st.cor[2]), gd2);
     const ff t1 = ff_add(du1, u1), t2 = ff_add(du2, u2);
     solve(gk, c, t1, r1, t2, r2, G1, G2, G3, dl);
     if (NEEDF) {
@@ -288,15 +289,18 @@ PF_FF_FN MichaelisFast::Gk fast_scaled(const Th& T, const MichaelisFast::Fk& k, 
 }
 
 // What a particle carries from substep to substep.
-//   x, h1, h2 with float carries cx, c1, c2: x_n, x_{n-1}, x_{n-2}
-//   BDF: a = x - h1, b = h1 - h2 in double, fa, fb the same in ff; fc = f(x_n)
-//   Adams: a, b = f_n, f_{n-1} in double with carries ca, cb; fa, fb, fc in ff
+//   x with float carry cx: x_n (Adams: h1, h2 with c1, c2: x_{n-1}, x_{n-2})
+//   a + ra, b + rb: the double and ff parts of what R multiplies: BDF x_n - x_{n-1}
+//   and x_{n-1} - x_{n-2} (the leading float of the increment and the rest, which
+//   spares an FP64 difference), Adams f_n and f_{n-1} (all but a float)
+//   fa, fb, fc: BDF x_n - x_{n-1}, x_{n-1} - x_{n-2}, f(x_n) in ff; Adams f_n, f_{n-1},
+//   f_{n-2}
 //   E: the error sums at 2^80 of their value
 struct FastCarry {
   double x[3], h1[3], h2[3];
   float cx[3], c1[3], c2[3];
   double a[3], b[3];
-  float ca[3], cb[3];
+  ff ra[3], rb[3];
   ff fa[3], fb[3], fc[3], E[3];
 };
 
@@ -307,7 +311,6 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
   const typename MF::Gk gk = fast_scaled(T, fk, c);
   ff P[3], Dv[3], xf[3];
   FastState st;
-  double R64[3];
   for (int i = 0; i < 3; ++i) {
     xf[i] = ff_from(w.x[i]);
     xf[i].l = f_add(xf[i].l, w.cx[i]);
@@ -326,20 +329,22 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
     for (int it = 0; it + 1 < K; ++it) MF::template early<FAM == 2>(fk, gk, c, xf, R, Dv);
   }
   for (int i = 0; i < 3; ++i) {
-    st.hh[i] = Dv[i].h;
-    const double hd = d_from_f(st.hh[i]);
+    const double hd = d_from_f(Dv[i].h);
     st.y[i] = w.x[i] + hd;
-    R64[i] = fma(c.ra, w.a[i], FAM != 0 ? fma(c.rb, w.b[i], hd) : hd);
-    // carries: x is w.x + cx, so the point's increment is hh - cx; a and b
-    // likewise have parts below their doubles
-    float r = f_fma(c.fra.h, w.ca[i], -w.cx[i]);
-    if (FAM != 0) r = f_fma(c.frb.h, w.cb[i], r);
-    if (FAM != 2) r = f_fma(-c.er, xf[i].h, r);
-    st.cor[i] = r;
+    st.R64[i] = fma(c.ra, w.a[i], FAM != 0 ? fma(c.rb, w.b[i], hd) : hd);
+    // the rest of R, what x is above w.x (its carry) and the weights' defect
+    if (FAM == 2) {
+      st.cor[i] = ff{f_fma(c.frb.h, w.rb[i].h, f_fma(c.fra.h, w.ra[i].h, -w.cx[i])), 0.0f};
+    } else {
+      ff r = ff_mul_raw(c.fra, w.ra[i]);
+      if (FAM == 1) r = ff_fma(c.frb, w.rb[i], r);
+      r.l = f_add(r.l, f_fma(-c.er, xf[i].h, -w.cx[i]));
+      st.cor[i] = r;
+    }
   }
   ff dl[3], dfy[3];
   double fy[3];
-  MF::template last<FAM != 0>(T, fk, gk, c, st, R64, dl, fy, dfy);
+  MF::template last<FAM != 0>(T, fk, gk, c, st, dl, fy, dfy);
   // every value finite and the last correction small: |d| <= 2^-4 |y|
   const float my = fabsf(f_from(st.y[0])) + fabsf(f_from(st.y[1])) + fabsf(f_from(st.y[2]));
   const float md = fabsf(dl[0].h) + fabsf(dl[1].h) + fabsf(dl[2].h);
@@ -348,7 +353,8 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
     const double xn = st.y[i] + d_from_f(dl[i].h);
     const float cn = dl[i].l;
     // the increment from x_n to the new state
-    const ff Dn = ff_add(ff_add(dl[i], st.hh[i]), -w.cx[i]);
+    const ff rest = ff_add(dl[i], -w.cx[i]);
+    const ff Dn = ff_add(rest, Dv[i].h);
     if (ERR) {
       const ff e = ff_mul(c.mus, ff_sub(Dn, P[i]));
       w.E[i] = ff_fma(e, e, w.E[i]);
@@ -357,30 +363,47 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
       w.fc[i] = w.fb[i];
       w.fb[i] = w.fa[i];
       w.b[i] = w.a[i];
-      w.cb[i] = w.ca[i];
+      w.rb[i] = w.ra[i];
       w.a[i] = fy[i] + d_from_f(dfy[i].h);
-      w.ca[i] = dfy[i].l;
+      w.ra[i] = ff{dfy[i].l, 0.0f};
       w.fa[i] = ff_from(w.a[i]);
-      w.fa[i].l = f_add(w.fa[i].l, w.ca[i]);
+      w.fa[i].l = f_add(w.fa[i].l, dfy[i].l);
     } else {
       if (FAM == 1) {
         w.b[i] = w.a[i];
-        w.cb[i] = w.ca[i];
+        w.rb[i] = w.ra[i];
         w.fc[i] = ff_add(ff_from(fy[i]), dfy[i]);
       }
       w.fb[i] = w.fa[i];
       w.fa[i] = Dn;
-      w.a[i] = xn - w.x[i];
-      w.ca[i] = f_sub(cn, w.cx[i]);
+      w.a[i] = d_from_f(Dv[i].h);
+      w.ra[i] = rest;
     }
-    w.h2[i] = w.h1[i];
-    w.c2[i] = w.c1[i];
-    w.h1[i] = w.x[i];
-    w.c1[i] = w.cx[i];
+    if (FAM == 2) {
+      w.h2[i] = w.h1[i];
+      w.c2[i] = w.c1[i];
+      w.h1[i] = w.x[i];
+      w.c1[i] = w.cx[i];
+    }
     w.x[i] = xn;
     w.cx[i] = cn;
   }
   return true;
+}
+
+PF_FF_FN double ff_value(ff a) { return (double)a.h + (double)a.l; }
+
+// x_n, x_{n-1}, x_{n-2} of component i as doubles (the BDF past from the increments).
+template <int FAM>
+PF_FF_FN void fast_history(const FastCarry& w, int i, double& x, double& h1, double& h2) {
+  x = w.x[i] + (double)w.cx[i];
+  if (FAM == 2) {
+    h1 = w.h1[i] + (double)w.c1[i];
+    h2 = w.h2[i] + (double)w.c2[i];
+  } else {
+    h1 = x - (w.a[i] + ff_value(w.ra[i]));
+    h2 = h1 - ff_value(w.fb[i]);
+  }
 }
 
 }  // namespace pfg

@@ -143,8 +143,8 @@ __device__ __forceinline__ int fast_run(const typename M::Th& T, const StepCoef*
     w.x[i] = x[i];
     w.h1[i] = h1[i];
     w.h2[i] = h2[i];
-    w.cx[i] = w.c1[i] = w.c2[i] = w.ca[i] = w.cb[i] = 0.0f;
-    w.E[i] = w.fc[i] = ff{0.0f, 0.0f};
+    w.cx[i] = w.c1[i] = w.c2[i] = 0.0f;
+    w.E[i] = w.fc[i] = w.ra[i] = w.rb[i] = ff{0.0f, 0.0f};
     if constexpr (FAM == 2) {
       w.a[i] = f0[i];
       w.b[i] = f1[i];
@@ -167,14 +167,12 @@ __device__ __forceinline__ int fast_run(const typename M::Th& T, const StepCoef*
     if (!fast_step<MF, FAM, ERR>(T, fk, fc[s], K, w)) break;
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    x[i] = w.x[i] + (double)w.cx[i];
-    h1[i] = w.h1[i] + (double)w.c1[i];
-    h2[i] = w.h2[i] + (double)w.c2[i];
-    if (ERR) E[i] = fma((double)w.E[i].h + (double)w.E[i].l, kErrUnscale, E[i]);
+    fast_history<FAM>(w, i, x[i], h1[i], h2[i]);
+    if (ERR) E[i] = fma(ff_value(w.E[i]), kErrUnscale, E[i]);
     if constexpr (FAM == 2) {
-      f0[i] = w.a[i] + (double)w.ca[i];
-      f1[i] = w.b[i] + (double)w.cb[i];
-      f2[i] = (double)w.fc[i].h + (double)w.fc[i].l;
+      f0[i] = w.a[i] + ff_value(w.ra[i]);
+      f1[i] = w.b[i] + ff_value(w.rb[i]);
+      f2[i] = ff_value(w.fc[i]);
     }
   }
   return s;

@@ -40,10 +40,8 @@ int interval(const Th& T, const Row* rows, int S, int K, double* s, double* E) {
   for (; n < S; ++n)
     if (!fast_step<MF, FAM, true>(T, fk, fast_coef(rows[n]), K, w)) break;
   for (int i = 0; i < 3; ++i) {
-    s[i] = w.x[i] + (double)w.cx[i];
-    s[3 + i] = w.h1[i] + (double)w.c1[i];
-    s[6 + i] = w.h2[i] + (double)w.c2[i];
-    E[i] = ((double)w.E[i].h + (double)w.E[i].l) * kErrUnscale;
+    fast_history<FAM>(w, i, s[i], s[3 + i], s[6 + i]);
+    E[i] = ff_value(w.E[i]) * kErrUnscale;
   }
   return n;
 }
