@@ -212,6 +212,7 @@ __device__ __forceinline__ void propagate(const typename M::Th& T, const StepCoe
 #pragma unroll
       for (int i = 0; i < D; ++i) f2[i] = f1[i];
   }
+  typename M::Cache cache;
   int s = 0;
 #pragma unroll 1
   for (int pass = 0; pass < (kFast ? 2 : 1); ++pass) {
@@ -255,7 +256,7 @@ __device__ __forceinline__ void propagate(const typename M::Th& T, const StepCoe
           }
         }
         if constexpr (M::kForced) r[0] = fma(c.gamma, c.in1, r[0]);
-        M::newton(T, c.gamma, r, y, K);
+        M::newton(T, c.gamma, r, y, K, c.ref, cache);
         if (ERR) {
 #pragma unroll
           for (int i = 0; i < D; ++i) {
@@ -276,7 +277,7 @@ __device__ __forceinline__ void propagate(const typename M::Th& T, const StepCoe
 #pragma unroll
           for (int i = 0; i < D; ++i) rr[i] = r[i];
           if constexpr (M::kForced) rr[0] = fma(c.gamma, c.in1, rr[0]);
-          M::newton(T, c.gamma, rr, y, K);
+          M::newton(T, c.gamma, rr, y, K, c.ref, cache);
         }
         feval<M>(T, c.in1, y, fn);
         if (ERR) {
