@@ -18,21 +18,20 @@
 //     and solves in ff: its correction is small beside y, so 2^-46 of it is
 //     below y's last bit, and so is what FP32 made of the point, since G is
 //     evaluated at the point itself.
-// The state stays a double plus a float carry (the low part of the last
-// correction, below the double's last bits), and Milne's estimate comes from
+// The state stays the double of the last iteration's point plus that iteration's
+// correction in ff, so a substep rounds it once, and Milne's estimate comes from
 // D - P without the cancellation of y - x_p.  The result is the K-th Newton
 // iterate to FP64 rounding, as before; a substep that does not satisfy this
 // reasoning (a non-finite value, a last correction that is not small, an
 // exponent outside the floats') is left to the FP64 path by fast_run's caller.
 //
-// A Robertson BDF2 substep with error sums takes 18 FP64 instructions instead
-// of 89, an M1 one 22 instead of 186.  Measured (GB300, device time):
-// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.275 ms, stage 2 1.08 -> 0.319 ms;
-// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.072 and 0.23 -> 0.085 ms (the exponentials and
-// roots of pf_math.cuh and the register bounds included).  The FP64 pipe is still
-// about 80 % busy, the issue slots 55 %.  Accuracy over an interval, against
-// quadruple precision on 200 particles of the prior, 2-norm of the state:
-// Robertson 2e-16 (plain FP64 9e-16), M1 2e-16 (4e-16).
+// A Robertson BDF2 substep with error sums takes 15 FP64 instructions instead
+// of 89, an M1 one 19 instead of 186.  Measured (GB300, device time):
+// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.262 ms, stage 2 1.08 -> 0.311 ms;
+// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.072 and 0.23 -> 0.084 ms (the exponentials and
+// roots of pf_math.cuh and the register bounds included).  Accuracy over an interval,
+// against quadruple precision on 200 particles of the prior, 2-norm of the state:
+// Robertson 3e-17 (plain FP64 9e-16), M1 6e-17 (4e-16).
 #pragma once
 #include "pf_ff.cuh"
 
@@ -289,7 +288,8 @@ PF_FF_FN MichaelisFast::Gk fast_scaled(const Th& T, const MichaelisFast::Fk& k, 
 }
 
 // What a particle carries from substep to substep.
-//   x with float carry cx: x_n (Adams: h1, h2 with c1, c2: x_{n-1}, x_{n-2})
+//   x + cx: x_n, the last iteration's point and its correction (Adams: h1 + c1, h2 +
+//   c2: x_{n-1}, x_{n-2})
 //   a + ra, b + rb: the double and ff parts of what R multiplies: BDF x_n - x_{n-1}
 //   and x_{n-1} - x_{n-2} (the leading float of the increment and the rest, which
 //   spares an FP64 difference), Adams f_n and f_{n-1} (all but a float)
@@ -298,7 +298,7 @@ PF_FF_FN MichaelisFast::Gk fast_scaled(const Th& T, const MichaelisFast::Fk& k, 
 //   E: the error sums at 2^80 of their value
 struct FastCarry {
   double x[3], h1[3], h2[3];
-  float cx[3], c1[3], c2[3];
+  ff cx[3], c1[3], c2[3];
   double a[3], b[3];
   ff ra[3], rb[3];
   ff fa[3], fb[3], fc[3], E[3];
@@ -312,8 +312,7 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
   ff P[3], Dv[3], xf[3];
   FastState st;
   for (int i = 0; i < 3; ++i) {
-    xf[i] = ff_from(w.x[i]);
-    xf[i].l = f_add(xf[i].l, w.cx[i]);
+    xf[i] = ff_add(ff_from(w.x[i]), w.cx[i]);
     ff p = ff_mul_raw(c.pa, w.fa[i]);
     p = ff_fma(c.pb, w.fb[i], p);
     if (FAM != 0) p = ff_fma(c.pc, w.fc[i], p);
@@ -328,19 +327,20 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
     }
     for (int it = 0; it + 1 < K; ++it) MF::template early<FAM == 2>(fk, gk, c, xf, R, Dv);
   }
+  float hh[3];
   for (int i = 0; i < 3; ++i) {
-    const double hd = d_from_f(Dv[i].h);
+    // the point x + hh, hh the float nearest D + cx: from x_n it is hh - cx
+    hh[i] = ff_add(Dv[i], w.cx[i]).h;
+    const double hd = d_from_f(hh[i]);
     st.y[i] = w.x[i] + hd;
     st.R64[i] = fma(c.ra, w.a[i], FAM != 0 ? fma(c.rb, w.b[i], hd) : hd);
-    // the rest of R, what x is above w.x (its carry) and the weights' defect
-    if (FAM == 2) {
-      st.cor[i] = ff{f_fma(c.frb.h, w.rb[i].h, f_fma(c.fra.h, w.ra[i].h, -w.cx[i])), 0.0f};
-    } else {
-      ff r = ff_mul_raw(c.fra, w.ra[i]);
-      if (FAM == 1) r = ff_fma(c.frb, w.rb[i], r);
-      r.l = f_add(r.l, f_fma(-c.er, xf[i].h, -w.cx[i]));
-      st.cor[i] = r;
-    }
+    // the rest: R's, the carry and the weights' defect
+    ff r{f_mul(c.fra.h, w.ra[i].h), 0.0f};
+    if (FAM == 2) r.h = f_fma(c.frb.h, w.rb[i].h, r.h);
+    else r = ff_mul_raw(c.fra, w.ra[i]);
+    if (FAM == 1) r = ff_fma(c.frb, w.rb[i], r);
+    if (FAM != 2) r.l = f_fma(-c.er, xf[i].h, r.l);
+    st.cor[i] = ff_sub(r, w.cx[i]);
   }
   ff dl[3], dfy[3];
   double fy[3];
@@ -350,11 +350,9 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
   const float md = fabsf(dl[0].h) + fabsf(dl[1].h) + fabsf(dl[2].h);
   if (!(md <= 0.0625f * my && my < 0x1.0p60f)) return false;
   for (int i = 0; i < 3; ++i) {
-    const double xn = st.y[i] + d_from_f(dl[i].h);
-    const float cn = dl[i].l;
     // the increment from x_n to the new state
-    const ff rest = ff_add(dl[i], -w.cx[i]);
-    const ff Dn = ff_add(rest, Dv[i].h);
+    const ff rest = ff_sub(dl[i], w.cx[i]);
+    const ff Dn = ff_add(rest, hh[i]);
     if (ERR) {
       const ff e = ff_mul(c.mus, ff_sub(Dn, P[i]));
       w.E[i] = ff_fma(e, e, w.E[i]);
@@ -376,7 +374,7 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
       }
       w.fb[i] = w.fa[i];
       w.fa[i] = Dn;
-      w.a[i] = d_from_f(Dv[i].h);
+      w.a[i] = d_from_f(hh[i]);
       w.ra[i] = rest;
     }
     if (FAM == 2) {
@@ -385,8 +383,8 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
       w.h1[i] = w.x[i];
       w.c1[i] = w.cx[i];
     }
-    w.x[i] = xn;
-    w.cx[i] = cn;
+    w.x[i] = st.y[i];
+    w.cx[i] = dl[i];
   }
   return true;
 }
@@ -396,10 +394,10 @@ PF_FF_FN double ff_value(ff a) { return (double)a.h + (double)a.l; }
 // x_n, x_{n-1}, x_{n-2} of component i as doubles (the BDF past from the increments).
 template <int FAM>
 PF_FF_FN void fast_history(const FastCarry& w, int i, double& x, double& h1, double& h2) {
-  x = w.x[i] + (double)w.cx[i];
+  x = w.x[i] + ff_value(w.cx[i]);
   if (FAM == 2) {
-    h1 = w.h1[i] + (double)w.c1[i];
-    h2 = w.h2[i] + (double)w.c2[i];
+    h1 = w.h1[i] + ff_value(w.c1[i]);
+    h2 = w.h2[i] + ff_value(w.c2[i]);
   } else {
     h1 = x - (w.a[i] + ff_value(w.ra[i]));
     h2 = h1 - ff_value(w.fb[i]);

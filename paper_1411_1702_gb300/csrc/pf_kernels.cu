@@ -143,8 +143,7 @@ __device__ __forceinline__ int fast_run(const typename M::Th& T, const StepCoef*
     w.x[i] = x[i];
     w.h1[i] = h1[i];
     w.h2[i] = h2[i];
-    w.cx[i] = w.c1[i] = w.c2[i] = 0.0f;
-    w.E[i] = w.fc[i] = w.ra[i] = w.rb[i] = ff{0.0f, 0.0f};
+    w.cx[i] = w.c1[i] = w.c2[i] = w.E[i] = w.fc[i] = w.ra[i] = w.rb[i] = ff{0.0f, 0.0f};
     if constexpr (FAM == 2) {
       w.a[i] = f0[i];
       w.b[i] = f1[i];

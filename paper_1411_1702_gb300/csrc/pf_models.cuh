@@ -36,8 +36,7 @@ struct Linear2 {
   // back substitution, y = b i and one correction by the residual b - o y, which
   // leaves y's own rounding whatever the reciprocal i of the pivot o lacks.  So
   // the reciprocals of one substep serve all whose gamma differs by rounding
-  // (StepCoef::ref).  13 FP64 instructions a substep (with the history's 17) instead
-  // of 22 (26).
+  // (StepCoef::ref).  10 FP64 instructions a substep instead of 22.
   struct Cache {
     double i1, i2;
     int ref = -1;
