@@ -377,8 +377,9 @@ __device__ __forceinline__ unsigned br_step(const BrTheta& T, const BrPar& par, 
 #pragma unroll
     for (int k = 0; k < 4; ++k) P[k] = ff_from(h * f[k]);
   }
-  // finite, and the correction small
-  const bool ok = !far && md <= 0x1.0p-6f * my && my < 0x1.0p60f;
+  // finite, and the iterations settled (a single one: 2^-40 of it, after two FP32 solves,
+  // below the last bit)
+  const bool ok = !far && md <= (K > 1 ? 0x1.0p-20f : 0x1.0p-13f) * my && my < 0x1.0p60f;
   const unsigned bad = __ballot_sync(0xffffffffu, !ok);
   if (bad & ((threadIdx.x & 16u) ? 0xffff0000u : 0x0000ffffu)) return bad;
 #pragma unroll

@@ -155,6 +155,41 @@ def test_interval_against_extended(shim, problem, lmm, K):
             t, depth, hp2, hp1 = t1, dout, rows[-2]["h"], rows[-1]["h"]
 
 
+@pytest.mark.parametrize("lmm,K", [(W.LMM_BDF2, 4), (W.LMM_BDF2, 2), (W.LMM_BDF3, 4), (W.LMM_AM3, 4)])
+def test_unconverged_iterations_are_refused(shim, lmm, K):
+    """M1's first interval over the whole prior, where some particles' Newton iterations
+    have not settled after K: the increment form stops before a substep whose K-th
+    iterate it would not give.  The tolerance is test_interval_against_extended's."""
+    if np.finfo(LD).eps > 2.0 ** -62:
+        pytest.skip("no extended precision on this machine")
+    w = W.michaelis(T=1, lmm=lmm)
+    cfg, rng = oracle.make_config(w), np.random.default_rng(9)
+    fam = 2 if lmm > 10 else 1 if lmm == W.LMM_BDF3 else 0
+    tab, S, _ = oracle.build_substeps(cfg, 0.0, w.t_obs[0], 0, 0.0, 0.0)
+    rows = oracle.substep_dicts(tab, S)
+    cold = 0 if fam == 2 else sum(r["kind"] == 1 for r in rows)
+    done = 0
+    for _ in range(60):
+        th = np.exp(rng.uniform(np.log(w.prior_lo), np.log(w.prior_hi)))
+        x = np.array(w.x0, dtype=float)
+        head = oracle.propagate(w.ode, K, th, tab, cold, x, x, x, with_error=True) if cold else (x, x, x, np.zeros(3))
+        f = [oracle.ode_f(w.ode, th, head[0], rows[cold]["tn"])] * 3
+        s, E, tht = np.concatenate([*head[:3], *f]), np.zeros(3), np.ascontiguousarray(th)
+        tbl = np.array([[r["kind"], r["gamma"], *((r["beta"][1], r["beta"][2], 0.0, *r["bab"][:3], 0.0) if fam == 2
+                         else (r["rho1"], r["rho2"], r["rho3"], r["pi0"], r["pi1"], r["pi2"], r["pi3"])),
+                         r["mu"], oracle.mm_input(r["t"])] for r in rows[cold:]])
+        n = shim.shim_interval(1, fam, tht.ctypes.data, tbl.ctypes.data, S - cold, K, s.ctypes.data, E.ctypes.data)
+        if n == 0:
+            continue
+        ref = _extended("michaelis", th, rows[:cold + n], K, x, x, x)
+        tol = 16 * S * 2.0 ** -53 * np.max(np.abs(ref[0]))
+        for i in range(3):
+            assert np.max(np.abs(s[3 * i:3 * i + 3] - ref[i])) <= tol
+        done += n
+    # most of the substeps do settle (at K = 2 fewer)
+    assert done >= (30 if K == 4 else 5) * (S - cold)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("lmm", [W.LMM_BDF2, W.LMM_BDF3, W.LMM_AM2])
 @pytest.mark.parametrize("N,K,scale", [(33, 1, 1.0), (129, 3, 1.0), (65, 2, 2.0 ** 30)])
