@@ -901,14 +901,15 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
     });
     below(x0, dst.h1);
     below(xb, dst.h2);
-    double lwn = -CUDART_INF, bad = 0.0;
+    double lwn = -CUDART_INF;
+    bool bad = false;
     if (tid < PB && n0 + tid < N) {
       // Step 5: new log weight
       const int64_t n = n0 + tid;
       lwn = ad_loglik(fd, ep, sm + L.base + tid * L.per + L.F[0]) - fd.ll1[slot_of(tid)];
       if (!finite_bits(lwn)) {
         lwn = -CUDART_INF;
-        bad = 1.0;
+        bad = true;
       }
       dst.lw[n] = lwn;
     }

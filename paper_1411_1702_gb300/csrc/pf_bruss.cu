@@ -555,16 +555,17 @@ __device__ __forceinline__ void bstage2_body(const FilterDev& fd, const EpochPar
     }
   }
   // 5: new log weight
-  double lwn = br_loglik(fd, ep, x) - fd.ll1[l], bad = 0.0;
+  double lwn = br_loglik(fd, ep, x) - fd.ll1[l];
+  bool bad = false;
   if (!finite_bits(lwn)) {
     lwn = -CUDART_INF;
-    bad = 1.0;
+    bad = true;
   }
   if (live && g == 0) {
     dst.lw[n] = lwn;
   } else {
     lwn = -CUDART_INF;
-    bad = 0.0;
+    bad = false;
   }
   stage2_tail(fd, epoch, lwn, bad, vb, vg, s_red, s_flag);
 }

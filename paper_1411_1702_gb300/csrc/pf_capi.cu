@@ -484,6 +484,7 @@ pf_status filter_create(pf_ode ode, int d, int p, int64_t N, pf_lmm lmm, double 
   fd.Ntile = shard_total > 0 ? shard_total : N;
   fd.shard_sums = nullptr;
   fd.sms = device_sms();
+  fd.scan_items = scan_items(fd.Ntile, fd.sms);
   f->shard_total = shard_total;
   f->shard_first = shard_first;
   f->shard_tiles_all = shard_total > 0 ? scan_tile_count(shard_total, fd.sms) : 0;

@@ -75,12 +75,12 @@ __device__ __forceinline__ void factor_covariance(const FilterDev& fd, int p, do
 __device__ __forceinline__ void stage1_tail(const FilterDev& fd, uint32_t epoch, double lg, int vb,
                                             int vg, double* s_red, int* s_flag) {
   Ctrl* ctrl = fd.ctrl;
-  const double bm = block_max(lg, s_red);
+  const double bm = block_max(order_key(lg), s_red);
   if (threadIdx.x == 0) fd.blk[vb] = bm;
   if (elect_last_block(fd.ticket + 0, s_flag, (unsigned)vg)) {
-    double m = -CUDART_INF;
-    for (int b = threadIdx.x; b < vg; b += blockDim.x) m = fmax(m, __ldcg(fd.blk + b));
-    m = block_max(m, s_red);
+    long long k = kKeyNegInf;
+    for (int b = threadIdx.x; b < vg; b += blockDim.x) k = max_key(k, __ldcg(fd.blk + b));
+    const double m = block_max(k, s_red);
     if (threadIdx.x == 0) {
       ctrl->lg_max = m;
       ctrl->n_unique = 0;
@@ -97,19 +97,19 @@ __device__ __forceinline__ void stage1_tail(const FilterDev& fd, uint32_t epoch,
 // of zero-weight particles; the last of the filter's vg blocks stores the
 // maximum and flags a degenerate epoch.  Every thread of the block must call it.
 __device__ __forceinline__ void stage2_tail(const FilterDev& fd, uint32_t epoch, double lwn,
-                                            double bad, int vb, int vg, double* s_red, int* s_flag) {
+                                            bool bad, int vb, int vg, double* s_red, int* s_flag) {
   Ctrl* ctrl = fd.ctrl;
-  const double bm = block_max(lwn, s_red);
-  const double nb = block_sum(bad, s_red);
+  const double bm = block_max(order_key(lwn), s_red);
+  const int nb = __syncthreads_count(bad);
   if (threadIdx.x == 0) {
     fd.blk[vb] = bm;
-    if (nb > 0.0)
+    if (nb > 0)
       atomicAdd(reinterpret_cast<unsigned long long*>(&ctrl->n_nonfinite), (unsigned long long)nb);
   }
   if (elect_last_block(fd.ticket + 2, s_flag, (unsigned)vg)) {
-    double m = -CUDART_INF;
-    for (int b = threadIdx.x; b < vg; b += blockDim.x) m = fmax(m, __ldcg(fd.blk + b));
-    m = block_max(m, s_red);
+    long long k = kKeyNegInf;
+    for (int b = threadIdx.x; b < vg; b += blockDim.x) k = max_key(k, __ldcg(fd.blk + b));
+    const double m = block_max(k, s_red);
     if (threadIdx.x == 0) {
       ctrl->lw_max = m;
       if (!(m > -CUDART_INF)) {

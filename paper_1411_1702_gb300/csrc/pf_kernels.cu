@@ -390,7 +390,7 @@ __device__ __forceinline__ void stage1_body(const FilterDev& fd, const EpochPara
 // its readers apply the tile offsets and floors (CumTiles).
 __device__ __forceinline__ ScanArgs scan_args(const FilterDev& fd) {
   Ctrl* ctrl = fd.ctrl;
-  return ScanArgs{fd.lg, fd.N, fd.Ntile, fd.sms, ctrl->lg_max, fd.c, fd.blk, fd.boff, fd.pmax,
+  return ScanArgs{fd.lg, fd.N, fd.scan_items, ctrl->lg_max, fd.c, fd.blk, fd.boff, fd.pmax,
                   fd.ticket + 1, &ctrl->c_total};
 }
 
@@ -406,7 +406,7 @@ __device__ __forceinline__ void scan_tile_body(const FilterDev& fd, int vb, int 
 // The filter's cumulative weights as the tile pass leaves them: the offsets
 // and floors are applied on read (no separate offset pass over c).
 __device__ __forceinline__ CumTiles cum_tiles(const FilterDev& fd) {
-  return CumTiles{fd.c, fd.boff, fd.pmax, (uint32_t)scan_tile_len(fd.Ntile, fd.sms)};
+  return CumTiles{fd.c, fd.boff, fd.pmax, (uint32_t)(kScanThreads * fd.scan_items)};
 }
 
 __device__ __forceinline__ double resample_u(const FilterDev& fd, const EpochParams* __restrict__ ep) {
@@ -442,7 +442,7 @@ __device__ __forceinline__ void stage2_body(const FilterDev& fd, const EpochPara
   const uint32_t epoch = ep->epoch;
   const int64_t n = (int64_t)vb * blockDim.x + threadIdx.x;
   double lwn = -CUDART_INF;
-  double bad = 0.0;
+  bool bad = false;
   if (n < N) {
     const int64_t l = fd.idx[n];
     // 4a: phi_{j+1} = (a phi^l + (1 - a) phibar) + s L z
@@ -495,7 +495,7 @@ __device__ __forceinline__ void stage2_body(const FilterDev& fd, const EpochPara
     lwn = ll2 - fd.ll1[l];
     if (!finite_bits(lwn)) {
       lwn = -CUDART_INF;
-      bad = 1.0;
+      bad = true;
     }
 #pragma unroll
     for (int i = 0; i < D; ++i) {
@@ -687,11 +687,17 @@ __device__ __forceinline__ void moments_commit(const FilterDev& fd, int is_init,
   // statistics and warp 2 the state mean.
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const double S0 = s_tot[Lay::kS0];
+  // each warp's divisions and the logarithm before the barrier, side by side
+  double inv = 0.0, ess = 0.0, logW = 0.0;
+  if (wid == 0 || wid == 2) inv = 1.0 / S0;
+  if (wid == 1) {
+    if (lane == 0) ess = S0 * S0 / s_tot[Lay::kW2];
+    if (lane == 1) logW = M + log(S0);
+  }
   double* s_m1 = s_part;                // P values
   double* s_C = s_part + kPMax;         // kPMax^2 values
   constexpr int NC = P * (P + 1) / 2;
   if (wid == 0) {
-    const double inv = 1.0 / S0;
     bool bad = !(S0 > 0.0);
     if (lane < kPMax * kPMax) s_C[lane] = 0.0;
     if (lane < P) {
@@ -730,13 +736,12 @@ __device__ __forceinline__ void moments_commit(const FilterDev& fd, int is_init,
   } else if (wid == 1) {
     if (lane == 0) {
       ctrl->wsum = S0;
-      ctrl->ess = S0 * S0 / s_tot[Lay::kW2];
-      ctrl->logW = M + log(S0);
+      ctrl->ess = ess;
       ctrl->cur = 1 - cur;
       if (!is_init) ctrl->epochs_done += 1;
     }
+    if (lane == 1) ctrl->logW = logW;
   } else if (wid == 2) {
-    const double inv = 1.0 / S0;
     for (int i = lane; i < D; i += 32) fd.xbar[i] = s_tot[Lay::kSx + i] * inv;
   }
 }
@@ -989,7 +994,8 @@ __global__ void __launch_bounds__(kScanThreads) k_batch_scan_tile(const FilterDe
   const BatchTile t = tiles[blockIdx.x];
   const FilterDev& fd = *(fds + t.f);
   if (fd.ctrl->status != PF_OK) return;
-  scan_tile_body(fd, t.vb, scan_tile_count(fd.N, fd.sms), s_warp, &s_flag);
+  const uint32_t len = (uint32_t)(kScanThreads * fd.scan_items);
+  scan_tile_body(fd, t.vb, (int)(((uint32_t)fd.N + len - 1) / len), s_warp, &s_flag);
 }
 
 __global__ void __launch_bounds__(kResampleThreads) k_batch_resample(

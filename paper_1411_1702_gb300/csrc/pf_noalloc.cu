@@ -72,36 +72,36 @@ __global__ void __launch_bounds__(kNaThreads) k_na_max(const double* __restrict_
                                                      NaScratch sc) {
   __shared__ double s_red[32];
   __shared__ int s_flag;
-  double m = -CUDART_INF;
+  long long key = kKeyNegInf;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N;
        k += (int64_t)gridDim.x * blockDim.x)
-    if (finite_bits(lg[k])) m = fmax(m, lg[k]);
-  m = block_max(m, s_red);
+    if (finite_bits(lg[k])) key = max_key(key, lg[k]);
+  const double m = block_max(key, s_red);
   if (threadIdx.x == 0) sc.blockmax[blockIdx.x] = m;
   if (elect_last_block(sc.ticket + 0, &s_flag, gridDim.x)) {
-    double t = -CUDART_INF;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) t = fmax(t, __ldcg(sc.blockmax + b));
-    t = block_max(t, s_red);
+    key = kKeyNegInf;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) key = max_key(key, __ldcg(sc.blockmax + b));
+    const double t = block_max(key, s_red);
     if (threadIdx.x == 0) sc.head[0] = t;
   }
 }
 
 // the filter's scan (scan_tile_core, scan_add_core) on the caller's buffers
-__device__ __forceinline__ ScanArgs na_scan_args(const double* lg, int64_t N, int sms, double* c,
+__device__ __forceinline__ ScanArgs na_scan_args(const double* lg, int64_t N, int items, double* c,
                                                  const NaScratch& sc) {
-  return ScanArgs{lg, N, N, sms, __ldcg(sc.head), c, sc.tile, sc.boff, sc.pmax, sc.ticket + 1, nullptr};
+  return ScanArgs{lg, N, items, __ldcg(sc.head), c, sc.tile, sc.boff, sc.pmax, sc.ticket + 1, nullptr};
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_na_scan_tile(const double* __restrict__ lg,
-                                                             int64_t N, int sms, double* c,
+                                                             int64_t N, int items, double* c,
                                                              NaScratch sc) {
   __shared__ double s_warp[33];
   __shared__ int s_flag;
-  scan_tile_core(na_scan_args(lg, N, sms, c, sc), blockIdx.x, gridDim.x, s_warp, &s_flag);
+  scan_tile_core(na_scan_args(lg, N, items, c, sc), blockIdx.x, gridDim.x, s_warp, &s_flag);
 }
 
-__global__ void __launch_bounds__(256) k_na_scan_add(int64_t N, int sms, double* c, NaScratch sc) {
-  scan_add_core(na_scan_args(nullptr, N, sms, c, sc), (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+__global__ void __launch_bounds__(256) k_na_scan_add(int64_t N, int items, double* c, NaScratch sc) {
+  scan_add_core(na_scan_args(nullptr, N, items, c, sc), (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // the filter's merge-path search (resample_tile), one block per diagonal tile;
@@ -167,7 +167,7 @@ extern "C" pf_status pf_resample_systematic_noalloc(const double* log_g, int64_t
   }
   // a second line of defence behind the static_asserts: the layout must hold
   // this N's tiles and corners on this device
-  const int sms = device_sms();
+  const int sms = device_sms(), items = scan_items(N, sms);
   if (scan_tile_count(N, sms) > kNaMaxTiles || rs_tiles(N) + 1 > kNaMaxCorners) {
     set_thread_error("pf_resample_systematic_noalloc: scratch layout too small for this N");
     return PF_ERR_BUDGET;
@@ -188,8 +188,8 @@ extern "C" pf_status pf_resample_systematic_noalloc(const double* log_g, int64_t
     const unsigned g_max = (unsigned)(mb < kNaMaxBlocks ? mb : kNaMaxBlocks);
     k_na_max<<<g_max, kNaThreads, 0, st>>>(log_g, N, sc);
     k_na_scan_tile<<<(unsigned)scan_tile_count(N, sms), kScanThreads, 0, st>>>(
-        log_g, N, sms, cumulative, sc);
-    k_na_scan_add<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(N, sms, cumulative, sc);
+        log_g, N, items, cumulative, sc);
+    k_na_scan_add<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(N, items, cumulative, sc);
     const bool two = rs_two_phase(N, sms);
     if (two) k_na_corners<<<rs_corner_blocks(N), 256, 0, st>>>(cumulative, N, u, sc.corners);
     k_na_resample<<<resample_blocks(N), kResampleThreads, 0, st>>>(cumulative, N, u, idx,

@@ -31,6 +31,7 @@ __device__ __forceinline__ double block_exclusive_scan(double v, double* s_warp,
     double wi = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
+      if (o >= nw) break;  // (adds nothing to the nw warps' totals)
       const double t = __shfl_up_sync(0xffffffffu, wi, o);
       if (lane >= o) wi = Op::apply(t, wi);
     }
@@ -140,9 +141,9 @@ struct MaxNonnegOp {
 struct ScanArgs {
   const double* lg;  // N log weights
   int64_t N;
-  int64_t Ntile;     // the ensemble size whose tile length applies (N, or the
-                     // whole ensemble's size for a shard of it)
-  int sms;           // the device's SM count (the tile length depends on it)
+  int items;         // values a thread: scan_items of the ensemble size whose tile length
+                     // applies (N, or the whole ensemble's for a shard of it) and the SM count,
+                     // formed on the host (its 64-bit divisions took every thread 0.7 us)
   double M;          // their maximum (the log-sum-exp shift)
   double* c;         // N cumulative weights (tile-local after the tile pass)
   double* tile;      // per-tile totals
@@ -184,7 +185,7 @@ __device__ __forceinline__ void scan_offsets_core(const double* tile, int nb, do
 // tile totals into offsets and floors.
 __device__ __forceinline__ void scan_tile_core(const ScanArgs& a, int vb, int vg, double* s_warp,
                                                int* s_flag) {
-  const int items = scan_items(a.Ntile, a.sms);
+  const int items = a.items;
   const int64_t base = (int64_t)vb * kScanThreads * items + (int64_t)threadIdx.x * items;
   double v[kScanItemsMax];
   double run = 0.0;
@@ -216,7 +217,7 @@ __device__ __forceinline__ void scan_tile_core(const ScanArgs& a, int vb, int vg
 // c_k = max(tile offset + tile-local sum, tile floor)
 __device__ __forceinline__ void scan_add_core(const ScanArgs& a, int64_t k) {
   if (k < a.N) {
-    const int64_t b = k / scan_tile_len(a.Ntile, a.sms);
+    const uint32_t b = (uint32_t)k / (uint32_t)(kScanThreads * a.items);
     a.c[k] = max_nonneg(__ldcg(a.boff + b) + a.c[k], __ldcg(a.pmax + b));
   }
 }
