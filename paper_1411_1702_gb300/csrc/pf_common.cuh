@@ -254,6 +254,25 @@ __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Launch kernel k on st with programmatic stream serialization: its blocks may
+// be scheduled while the stream's previous kernel drains, and the kernel's
+// pdl_wait() orders its accesses after that kernel's.
+template <typename... P, typename... A>
+static cudaError_t launch_pdl(void (*k)(P...), unsigned grid, unsigned block, size_t smem,
+                              cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Finite test on the bit pattern (integer pipe, no FP64 compare).
 __device__ __forceinline__ bool finite_bits(double v) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);

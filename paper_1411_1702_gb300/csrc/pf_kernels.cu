@@ -1122,25 +1122,6 @@ static void batch_stage_kernels(int lmm, BatchStageKernel& k1, BatchStageKernel&
   k2 = k_batch_stage<M, 2, kFamBdf12>;
 }
 
-// Launch kernel k on st with programmatic stream serialization: its blocks may
-// be scheduled while the stream's previous kernel drains, and the kernel's
-// pdl_wait() orders its accesses after that kernel's.
-template <typename... P, typename... A>
-static cudaError_t launch_pdl(void (*k)(P...), unsigned grid, unsigned block, size_t smem,
-                              cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, args...);
-}
-
 template <class M>
 static cudaError_t launch_epoch_t(const FilterDev& fd, const EpochParams* ep, int S,
                                   cudaStream_t st, cudaEvent_t* marks) {
