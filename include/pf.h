@@ -7,8 +7,10 @@
  * particle filter over (x, theta) whose particles are propagated by a linear
  * multistep method (BDF1-3, Adams-Moulton 1-3 with a full Newton solve per
  * particle and per substep, or Adams-Bashforth 1-3), and whose innovation
- * variance comes from the LMM's local error estimate (Step 4b).  All arithmetic is FP64 and runs in
- * hand-written CUDA kernels; nothing falls back to the CPU.
+ * variance comes from the LMM's local error estimate (Step 4b).  Results are FP64
+ * arithmetic's to rounding (the kernels work in doubles where their last bits count, in pairs of
+ * floats and scaled integers elsewhere).  Everything runs in hand-written CUDA kernels; nothing
+ * falls back to the CPU.
  *
  * Conventions
  *  - Every entry point returns a pf_status.  No C++ exception crosses the ABI.

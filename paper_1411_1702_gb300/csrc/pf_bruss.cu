@@ -20,7 +20,7 @@
 // to be exact beside the state, one step of refinement in ff follows.  A
 // particle the floats do not serve repeats the substep in FP64 on the same
 // lanes.  Measured (GB300, S = 20, stage 1 + stage 2): N = 1000 7.3 -> 0.22 ms,
-// N = 16384 8.57 -> 1.57 ms, N = 65536 23.4 -> 6.0 ms; the FP64 pipe is about half
+// N = 16384 8.57 -> 1.50 ms, N = 65536 23.4 -> 5.7 ms; the FP64 pipe is 60 %
 // busy, three warps a sub-partition (168 registers) waiting on each other's
 // results the rest; 128 registers (four warps, spills) and 64-thread blocks
 // changed the epochs by less than 4 %.
