@@ -14,10 +14,10 @@
 //     exact to 2^-47 of the terms (the Adams methods solve in ff: their
 //     explicit predictors are far off on stiff particles, where an inexact
 //     first step would be seen in the K-th);
-//   - the last evaluates G in FP64 at the point y = x_n + (leading float of D)
-//     and solves in ff: its correction is small beside y, so 2^-46 of it is
-//     below y's last bit, and so is what FP32 made of the point, since G is
-//     evaluated at the point itself.
+//   - the last evaluates G in FP64 at the point y = x_n + (leading float of D).
+//     Its correction is D's low float, known, plus a rest of about 2^-50 |y| that an
+//     FP32 solution serves; what FP32 made of the point does not matter, since G
+//     is evaluated at the point itself.  (A rest above 2^-34 |y| solves in ff.)
 // The state stays the double of the last iteration's point plus that iteration's
 // correction in ff, so a substep rounds it once, and Milne's estimate comes from
 // D - P without the cancellation of y - x_p.  The result is the K-th Newton
@@ -27,7 +27,7 @@
 //
 // A Robertson BDF2 substep with error sums takes 15 FP64 instructions instead
 // of 89, an M1 one 19 instead of 186.  Measured (GB300, device time):
-// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.262 ms, stage 2 1.08 -> 0.311 ms;
+// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.248 ms, stage 2 1.08 -> 0.294 ms;
 // M1 BDF2, N = 50000, S = 10: 0.16 -> 0.072 and 0.23 -> 0.084 ms (the exponentials and
 // roots of pf_math.cuh and the register bounds included).  Accuracy over an interval,
 // against quadruple precision on 200 particles of the prior, 2-norm of the state:
@@ -49,6 +49,10 @@ constexpr float kFastStepMin = 0x1.0p-60f, kFastStepMax = 0x1.0p40f;
 // the largest correction beside the state of a single iteration (its ff solve is good
 // to 2^-46); of the last of several: the models' kSettled
 constexpr float kFastSingle = 0x1.0p-7f;
+// The last correction is D's low floats lo, known, and a rest: an FP32 solution, good to
+// 2^-20, serves a rest of up to 2^-34 of the state.  It is below 2^-44 for 99.5 % of the
+// substeps of the prior (K = 2 and 4).
+constexpr float kFastRest = 0x1.0p-34f;
 
 // One substep's coefficients for the increment form (built in shared memory
 // from the StepCoef table by fast_coef):
@@ -90,7 +94,20 @@ PF_FF_FN FastCoef fast_coef(const C& c) {
 struct FastState {
   double y[3], R64[3];
   ff cor[3];
+  float lo[3];  // what D is above the point
 };
+
+// G + a, which nearly cancel
+PF_FF_FN float rest_of(ff G, float a) { return f_add(f_add(G.h, a), G.l); }
+
+// dl = lo + d unless d is too large beside the state for an FP32 solution
+PF_FF_FN bool rest_serves(const FastState& st, float y1, float y2, float y3, float d1, float d2, float d3,
+                          ff (&dl)[3]) {
+  dl[0] = two_sum(st.lo[0], d1);
+  dl[1] = two_sum(st.lo[1], d2);
+  dl[2] = two_sum(st.lo[2], d3);
+  return fabsf(d1) + fabsf(d2) + fabsf(d3) <= kFastRest * (fabsf(y1) + fabsf(y2) + fabsf(y3));
+}
 
 // ---------------------------------------------------------------- Robertson
 struct RobertsonFast {
@@ -125,6 +142,17 @@ struct RobertsonFast {
     dl[0] = ff_mul(im, ff_fma(q, dl[2], ff_sub(ff_mul(p, dl[1]), G1)));
   }
 
+  // the same in FP32; q, p, w as there
+  PF_FF_FN static void solve32(const Gk& k, float q, float p, float w, float G1, float G2, float G3, float& d1,
+                               float& d2, float& d3) {
+    const float im = f_rcp(k.op.h), l = f_mul(k.gk1.h, im);
+    const float den = f_fma(im, f_fma(q, w, p), f_add(1.0f, w));
+    const float num = f_fma(f_mul(q, im), G3, -f_fma(l, G1, G2));
+    d2 = f_mul(num, f_rcp(den));
+    d3 = f_fma(w, d2, -G3);
+    d1 = f_mul(im, f_fma(q, d3, f_fma(p, d2, -G1)));
+  }
+
   // G = D + R - gamma f at y = x + D, then D -= (I - gamma J)^{-1} G, in FP32
   // (WIDE: in ff)
   template <bool WIDE>
@@ -142,14 +170,8 @@ struct RobertsonFast {
       for (int i = 0; i < 3; ++i) Dv[i] = ff_add(Dv[i], dl[i]);
       return;
     }
-    const float G1 = g1.h, G2 = g2.h, G3 = g3.h;
-    const float p = f_mul(k.gk3.h, y3.h), w = f_add(t.h, t.h);
-    const float im = f_rcp(k.op.h), l = f_mul(k.gk1.h, im);
-    const float den = f_fma(im, f_fma(q.h, w, p), f_add(1.0f, w));
-    const float num = f_fma(f_mul(q.h, im), G3, -f_fma(l, G1, G2));
-    const float d2 = f_mul(num, f_rcp(den));
-    const float d3 = f_fma(w, d2, -G3);
-    const float d1 = f_mul(im, f_fma(q.h, d3, f_fma(p, d2, -G1)));
+    float d1, d2, d3;
+    solve32(k, q.h, f_mul(k.gk3.h, y3.h), f_add(t.h, t.h), g1.h, g2.h, g3.h, d1, d2, d3);
     Dv[0] = ff_add(Dv[0], d1);
     Dv[1] = ff_add(Dv[1], d2);
     Dv[2] = ff_add(Dv[2], d3);
@@ -167,9 +189,17 @@ struct RobertsonFast {
     const ff G1 = ff_add(ff_from(fma(c.gamma, s64, st.R64[0])), st.cor[0]);
     const ff G2 = ff_add(ff_from(fma(-c.gamma, s64, fma(c.gamma, c64, st.R64[1]))), st.cor[1]);
     const ff G3 = ff_add(ff_from(fma(-c.gamma, c64, st.R64[2])), st.cor[2]);
-    const ff f2 = ff_from(y2), f3 = ff_from(y3);
-    solve(k, f2, f3, G1, G2, G3, dl);
+    const float e1 = f_from(y1), e2f = f_from(y2), e3 = f_from(y3);
+    // G + (I - gamma J) lo: what the low floats leave to correct
+    const float q = f_mul(k.gk3.h, e2f), p = f_mul(k.gk3.h, e3), t = f_mul(k.gk2.h, e2f), w = f_add(t, t);
+    const float v = f_fma(k.gk1.h, st.lo[0], -f_fma(p, st.lo[1], f_mul(q, st.lo[2])));
+    const float wl = f_mul(w, st.lo[1]);
+    float d1, d2, d3;
+    solve32(k, q, p, w, rest_of(G1, f_add(st.lo[0], v)), rest_of(G2, f_add(f_sub(st.lo[1], v), wl)),
+            rest_of(G3, f_sub(st.lo[2], wl)), d1, d2, d3);
+    if (!rest_serves(st, e1, e2f, e3, d1, d2, d3, dl)) solve(k, ff_from(y2), ff_from(y3), G1, G2, G3, dl);
     if (NEEDF) {
+      const ff f2 = ff_from(y2), f3 = ff_from(y3);
       // f is quadratic: f(y + d) = f(y) + J d + Q(d, d), in ff beside FP64 f(y)
       const ff e2 = ff_add(f2, dl[1]);
       const ff dq = ff_add(ff_mul(f3, dl[1]), ff_mul(e2, dl[2]));      // y2 y3 changes by
@@ -229,6 +259,14 @@ struct MichaelisFast {
     dl[2] = ff_div(ff_sub(ff_mul(gb, dl[1]), G3), ff_one_plus(gk.gl));
   }
 
+  // the same in FP32; ga, gb = gamma u/s
+  PF_FF_FN static void solve32(const Gk& gk, float ga, float gb, float G1, float G2, float G3, float& d1,
+                               float& d2, float& d3) {
+    d1 = -f_mul(G1, f_rcp(f_add(1.0f, ga)));
+    d2 = f_mul(f_fma(ga, d1, -G2), f_rcp(f_add(1.0f, gb)));
+    d3 = f_mul(f_fma(gb, d2, -G3), f_rcp(f_add(1.0f, gk.gl.h)));
+  }
+
   template <bool WIDE>
   PF_FF_FN static void early(const Fk& k, const Gk& gk, const FastCoef& c, const ff (&x)[3],
                              const ff (&R)[3], ff (&Dv)[3]) {
@@ -247,11 +285,9 @@ struct MichaelisFast {
       for (int i = 0; i < 3; ++i) Dv[i] = ff_add(Dv[i], dl[i]);
       return;
     }
-    const float G1 = g1.h, G2 = g2.h, G3 = g3.h;
-    const float ga = f_mul(f_mul(c.g.h, u1.h), f_rcp(s1.h)), gb = f_mul(f_mul(c.g.h, u2.h), f_rcp(s2.h));
-    const float d1 = -f_mul(G1, f_rcp(f_add(1.0f, ga)));
-    const float d2 = f_mul(f_fma(ga, d1, -G2), f_rcp(f_add(1.0f, gb)));
-    const float d3 = f_mul(f_fma(gb, d2, -G3), f_rcp(f_add(1.0f, gk.gl.h)));
+    float d1, d2, d3;
+    solve32(gk, f_mul(f_mul(c.g.h, u1.h), f_rcp(s1.h)), f_mul(f_mul(c.g.h, u2.h), f_rcp(s2.h)), g1.h, g2.h,
+            g3.h, d1, d2, d3);
     Dv[0] = ff_add(Dv[0], d1);
     Dv[1] = ff_add(Dv[1], d2);
     Dv[2] = ff_add(Dv[2], d3);
@@ -274,9 +310,16 @@ struct MichaelisFast {
     const ff G1 = ff_sub(ff_add(ff_from(fma(-c.gamma, fy[0], st.R64[0])), st.cor[0]), gd1);
     const ff G2 = ff_sub(ff_add(ff_add(ff_from(fma(-c.gamma, fy[1], st.R64[1])), st.cor[1]), gd1), gd2);
     const ff G3 = ff_add(ff_add(ff_from(fma(-c.gamma, fy[2], st.R64[2])), st.cor[2]), gd2);
-    const ff t1 = ff_add(du1, u1), t2 = ff_add(du2, u2);
-    solve(gk, c, t1, r1, t2, r2, G1, G2, G3, dl);
+    // G + (I - gamma J) lo: what the low floats leave to correct
+    const float ga = f_mul(f_mul(c.g.h, u1), r1.h), gb = f_mul(f_mul(c.g.h, u2), r2.h);
+    const float al = f_mul(ga, st.lo[0]), bl = f_mul(gb, st.lo[1]);
+    float d1, d2, d3;
+    solve32(gk, ga, gb, rest_of(G1, f_add(st.lo[0], al)), rest_of(G2, f_sub(f_add(st.lo[1], bl), al)),
+            rest_of(G3, f_sub(f_fma(gk.gl.h, st.lo[2], st.lo[2]), bl)), d1, d2, d3);
+    const bool rest = rest_serves(st, f_from(st.y[0]), f_from(st.y[1]), f_from(st.y[2]), d1, d2, d3, dl);
+    if (!rest) solve(gk, c, ff_add(du1, u1), r1, ff_add(du2, u2), r2, G1, G2, G3, dl);
     if (NEEDF) {
+      const ff t1 = ff_add(du1, u1), t2 = ff_add(du2, u2);
       // u(s + d) = u - u d/(s + d)
       const ff v1 = ff_sub(du1, ff_div(ff_mul(t1, dl[0]), ff_add(e1, dl[0])));
       const ff v2 = ff_sub(du2, ff_div(ff_mul(t2, dl[1]), ff_add(e2, dl[1])));
@@ -339,7 +382,9 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
   float hh[3];
   for (int i = 0; i < 3; ++i) {
     // the point x + hh, hh the float nearest D + cx: from x_n it is hh - cx
-    hh[i] = ff_add(Dv[i], w.cx[i]).h;
+    const ff s = ff_add(Dv[i], w.cx[i]);
+    hh[i] = s.h;
+    st.lo[i] = s.l;
     const double hd = d_from_f(hh[i]);
     st.y[i] = w.x[i] + hd;
     st.R64[i] = fma(c.ra, w.a[i], FAM != 0 ? fma(c.rb, w.b[i], hd) : hd);
