@@ -8,12 +8,12 @@
 // has R = r-terms of the differences x_n - x_{n-1}, x_{n-1} - x_{n-2} (BDF) or of
 // the stored derivatives (Adams-Moulton), all small beside x_n, and the
 // predictor's increment P likewise.  Of the K Newton iterations
-//   - the first K - 1 evaluate G in ff (pf_ff.cuh) and solve their linear
-//     system in FP32: as with the unrefined reciprocals of the FP64 path, an
-//     inexact correction is repaired by the next iteration's residual, here
-//     exact to 2^-47 of the terms (the Adams methods solve in ff: their
-//     explicit predictors are far off on stiff particles, where an inexact
-//     first step would be seen in the K-th);
+//   - the first K - 1 solve their linear system in FP32: as with the unrefined
+//     reciprocals of the FP64 path, an inexact correction is repaired by the next
+//     iteration's residual.  The one before the last takes its residual in ff
+//     (pf_ff.cuh, sums not renormalised), those before it in FP32.  (The Adams methods
+//     evaluate and solve in ff: their explicit predictors are far off on stiff
+//     particles, where an inexact first step would be seen in the K-th.)
 //   - the last evaluates G in FP64 at the point y = x_n + (leading float of D).
 //     Its correction is D's low float, known, plus a rest of about 2^-50 |y| that an
 //     FP32 solution serves; what FP32 made of the point does not matter, since G
@@ -27,8 +27,8 @@
 //
 // A Robertson BDF2 substep with error sums takes 15 FP64 instructions instead
 // of 89, an M1 one 19 instead of 186.  Measured (GB300, device time):
-// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.248 ms, stage 2 1.08 -> 0.294 ms;
-// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.072 and 0.23 -> 0.084 ms (the exponentials and
+// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.234 ms, stage 2 1.08 -> 0.293 ms;
+// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.065 and 0.23 -> 0.077 ms (the exponentials and
 // roots of pf_math.cuh and the register bounds included).  Accuracy over an interval,
 // against quadruple precision on 200 particles of the prior, 2-norm of the state:
 // Robertson 3e-17 (plain FP64 9e-16), M1 6e-17 (4e-16).
@@ -158,23 +158,43 @@ struct RobertsonFast {
   template <bool WIDE>
   PF_FF_FN static void early(const Fk&, const Gk& k, const FastCoef&, const ff (&x)[3], const ff (&R)[3],
                              ff (&Dv)[3]) {
-    const ff y1 = ff_add(x[0], Dv[0]), y2 = ff_add(x[1], Dv[1]), y3 = ff_add(x[2], Dv[2]);
-    const ff q = ff_mul(k.gk3, y2), t = ff_mul(k.gk2, y2);
-    const ff ab = ff_sub(ff_mul(k.gk1, y1), ff_mul(q, y3));
-    const ff c = ff_mul(t, y2);
-    const ff g1 = ff_add(ff_add(Dv[0], R[0]), ab), g3 = ff_sub(ff_add(Dv[2], R[2]), c);
-    const ff g2 = ff_add(ff_sub(ff_add(Dv[1], R[1]), ab), c);
     if (WIDE) {
+      const ff y1 = ff_add(x[0], Dv[0]), y2 = ff_add(x[1], Dv[1]), y3 = ff_add(x[2], Dv[2]);
+      const ff ab = ff_sub(ff_mul(k.gk1, y1), ff_mul(ff_mul(k.gk3, y2), y3));
+      const ff c = ff_mul(ff_mul(k.gk2, y2), y2);
+      const ff g1 = ff_add(ff_add(Dv[0], R[0]), ab), g3 = ff_sub(ff_add(Dv[2], R[2]), c);
+      const ff g2 = ff_add(ff_sub(ff_add(Dv[1], R[1]), ab), c);
       ff dl[3];
       solve(k, y2, y3, g1, g2, g3, dl);
       for (int i = 0; i < 3; ++i) Dv[i] = ff_add(Dv[i], dl[i]);
       return;
     }
+    const ff y1 = ff_add_raw(x[0], Dv[0]), y2 = ff_add_raw(x[1], Dv[1]), y3 = ff_add_raw(x[2], Dv[2]);
+    const ff q = ff_mul_raw(k.gk3, y2), t = ff_mul_raw(k.gk2, y2);
+    const ff ab = ff_sub_raw(ff_mul_raw(k.gk1, y1), ff_mul_raw(q, y3));
+    const ff c = ff_mul_raw(t, y2);
+    const ff g1 = ff_add_raw(ff_add_raw(Dv[0], R[0]), ab), g3 = ff_sub_raw(ff_add_raw(Dv[2], R[2]), c);
+    const ff g2 = ff_add_raw(ff_sub_raw(ff_add_raw(Dv[1], R[1]), ab), c);
     float d1, d2, d3;
-    solve32(k, q.h, f_mul(k.gk3.h, y3.h), f_add(t.h, t.h), g1.h, g2.h, g3.h, d1, d2, d3);
+    solve32(k, q.h, f_mul(k.gk3.h, y3.h), f_add(t.h, t.h), f_add(g1.h, g1.l), f_add(g2.h, g2.l),
+            f_add(g3.h, g3.l), d1, d2, d3);
     Dv[0] = ff_add(Dv[0], d1);
     Dv[1] = ff_add(Dv[1], d2);
     Dv[2] = ff_add(Dv[2], d3);
+  }
+
+  // the same with the residual in FP32
+  PF_FF_FN static void first(const Fk&, const Gk& k, const FastCoef&, const ff (&x)[3], const ff (&R)[3],
+                             ff (&Dv)[3]) {
+    const float y1 = f_add(x[0].h, Dv[0].h), y2 = f_add(x[1].h, Dv[1].h), y3 = f_add(x[2].h, Dv[2].h);
+    const float q = f_mul(k.gk3.h, y2), t = f_mul(k.gk2.h, y2);
+    const float ab = f_fma(k.gk1.h, y1, -f_mul(q, y3)), c = f_mul(t, y2);
+    float d1, d2, d3;
+    solve32(k, q, f_mul(k.gk3.h, y3), f_add(t, t), f_add(f_add(Dv[0].h, R[0].h), ab),
+            f_add(f_sub(f_add(Dv[1].h, R[1].h), ab), c), f_sub(f_add(Dv[2].h, R[2].h), c), d1, d2, d3);
+    Dv[0] = ff{f_add(Dv[0].h, d1), 0.0f};
+    Dv[1] = ff{f_add(Dv[1].h, d2), 0.0f};
+    Dv[2] = ff{f_add(Dv[2].h, d3), 0.0f};
   }
 
   // the last iteration's correction.  fy, dfy: f at the corrected point (double
@@ -270,27 +290,51 @@ struct MichaelisFast {
   template <bool WIDE>
   PF_FF_FN static void early(const Fk& k, const Gk& gk, const FastCoef& c, const ff (&x)[3],
                              const ff (&R)[3], ff (&Dv)[3]) {
-    const ff s1 = ff_add(ff_add(x[0], Dv[0]), k.fk1), s2 = ff_add(ff_add(x[1], Dv[1]), k.fk2);
-    const ff y3 = ff_add(x[2], Dv[2]);
-    const ff u1 = ff_div(k.fvk1, s1), u2 = ff_div(k.fvk2, s2);
-    const ff f1 = ff_add(gk.ff0, u1);
-    const ff f2 = ff_add(ff_sub(k.fvd, u1), u2);
-    const ff f3 = ff_sub(ff_sub(k.fvc, u2), ff{0.5f * y3.h, 0.5f * y3.l});
-    const ff g1 = ff_sub(ff_add(Dv[0], R[0]), ff_mul(c.g, f1));
-    const ff g2 = ff_sub(ff_add(Dv[1], R[1]), ff_mul(c.g, f2));
-    const ff g3 = ff_sub(ff_add(Dv[2], R[2]), ff_mul(c.g, f3));
     if (WIDE) {
+      const ff s1 = ff_add(ff_add(x[0], Dv[0]), k.fk1), s2 = ff_add(ff_add(x[1], Dv[1]), k.fk2);
+      const ff y3 = ff_add(x[2], Dv[2]);
+      const ff u1 = ff_div(k.fvk1, s1), u2 = ff_div(k.fvk2, s2);
+      const ff f1 = ff_add(gk.ff0, u1);
+      const ff f2 = ff_add(ff_sub(k.fvd, u1), u2);
+      const ff f3 = ff_sub(ff_sub(k.fvc, u2), ff{0.5f * y3.h, 0.5f * y3.l});
+      const ff g1 = ff_sub(ff_add(Dv[0], R[0]), ff_mul(c.g, f1));
+      const ff g2 = ff_sub(ff_add(Dv[1], R[1]), ff_mul(c.g, f2));
+      const ff g3 = ff_sub(ff_add(Dv[2], R[2]), ff_mul(c.g, f3));
       ff dl[3];
       solve(gk, c, u1, ff_rcp(s1), u2, ff_rcp(s2), g1, g2, g3, dl);
       for (int i = 0; i < 3; ++i) Dv[i] = ff_add(Dv[i], dl[i]);
       return;
     }
+    const ff s1 = ff_add(ff_add_raw(x[0], Dv[0]), k.fk1), s2 = ff_add(ff_add_raw(x[1], Dv[1]), k.fk2);
+    const ff y3 = ff_add_raw(x[2], Dv[2]);
+    const ff u1 = ff_div(k.fvk1, s1), u2 = ff_div(k.fvk2, s2);
+    const ff f1 = ff_add_raw(gk.ff0, u1);
+    const ff f2 = ff_add_raw(ff_sub_raw(k.fvd, u1), u2);
+    const ff f3 = ff_sub_raw(ff_sub_raw(k.fvc, u2), ff{0.5f * y3.h, 0.5f * y3.l});
+    const ff g1 = ff_sub_raw(ff_add_raw(Dv[0], R[0]), ff_mul_raw(c.g, f1));
+    const ff g2 = ff_sub_raw(ff_add_raw(Dv[1], R[1]), ff_mul_raw(c.g, f2));
+    const ff g3 = ff_sub_raw(ff_add_raw(Dv[2], R[2]), ff_mul_raw(c.g, f3));
     float d1, d2, d3;
-    solve32(gk, f_mul(f_mul(c.g.h, u1.h), f_rcp(s1.h)), f_mul(f_mul(c.g.h, u2.h), f_rcp(s2.h)), g1.h, g2.h,
-            g3.h, d1, d2, d3);
+    solve32(gk, f_mul(f_mul(c.g.h, u1.h), f_rcp(s1.h)), f_mul(f_mul(c.g.h, u2.h), f_rcp(s2.h)),
+            f_add(g1.h, g1.l), f_add(g2.h, g2.l), f_add(g3.h, g3.l), d1, d2, d3);
     Dv[0] = ff_add(Dv[0], d1);
     Dv[1] = ff_add(Dv[1], d2);
     Dv[2] = ff_add(Dv[2], d3);
+  }
+
+  // the same with the residual in FP32
+  PF_FF_FN static void first(const Fk& k, const Gk& gk, const FastCoef& c, const ff (&x)[3], const ff (&R)[3],
+                             ff (&Dv)[3]) {
+    const float r1 = f_rcp(f_add(f_add(x[0].h, Dv[0].h), k.fk1.h)), r2 = f_rcp(f_add(f_add(x[1].h, Dv[1].h), k.fk2.h));
+    const float u1 = f_mul(k.fvk1.h, r1), u2 = f_mul(k.fvk2.h, r2), g = c.g.h;
+    const float f1 = f_add(gk.ff0.h, u1), f2 = f_add(f_sub(k.fvd.h, u1), u2);
+    const float f3 = f_fma(-0.5f, f_add(x[2].h, Dv[2].h), f_sub(k.fvc.h, u2));
+    float d1, d2, d3;
+    solve32(gk, f_mul(f_mul(g, u1), r1), f_mul(f_mul(g, u2), r2), f_fma(-g, f1, f_add(Dv[0].h, R[0].h)),
+            f_fma(-g, f2, f_add(Dv[1].h, R[1].h)), f_fma(-g, f3, f_add(Dv[2].h, R[2].h)), d1, d2, d3);
+    Dv[0] = ff{f_add(Dv[0].h, d1), 0.0f};
+    Dv[1] = ff{f_add(Dv[1].h, d2), 0.0f};
+    Dv[2] = ff{f_add(Dv[2].h, d3), 0.0f};
   }
 
   template <bool NEEDF, class Th>
@@ -365,6 +409,13 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
   FastState st;
   for (int i = 0; i < 3; ++i) {
     xf[i] = ff_add(ff_from(w.x[i]), w.cx[i]);
+    if (!ERR && FAM != 2) {
+      // a start for the iterations only: a float does
+      float p = f_fma(c.pb.h, w.fb[i].h, f_fma(c.pa.h, w.fa[i].h, f_mul(c.ep, xf[i].h)));
+      if (FAM == 1) p = f_fma(c.pc.h, w.fc[i].h, p);
+      Dv[i] = ff{p, 0.0f};
+      continue;
+    }
     ff p = ff_mul_raw(c.pa, w.fa[i]);
     p = ff_fma(c.pb, w.fb[i], p);
     if (FAM != 0) p = ff_fma(c.pc, w.fc[i], p);
@@ -377,7 +428,10 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
       R[i] = ff_mul(c.fra, w.fa[i]);
       if (FAM != 0) R[i] = ff_fma(c.frb, w.fb[i], R[i]);
     }
-    for (int it = 0; it + 1 < K; ++it) MF::template early<FAM == 2>(fk, gk, c, xf, R, Dv);
+    for (int it = 0; it + 1 < K; ++it) {
+      if (FAM != 2 && it + 2 < K) MF::first(fk, gk, c, xf, R, Dv);
+      else MF::template early<FAM == 2>(fk, gk, c, xf, R, Dv);
+    }
   }
   float hh[3];
   for (int i = 0; i < 3; ++i) {

@@ -91,6 +91,12 @@ PF_FF_FN ff ff_add(ff a, float b) {
   const ff s = two_sum(a.h, b);
   return fast_two_sum(s.h, f_add(s.l, a.l));
 }
+// a + b not renormalised (l up to h's size where they cancel), to 2^-45 of the larger
+PF_FF_FN ff ff_add_raw(ff a, ff b) {
+  const ff s = two_sum(a.h, b.h);
+  return ff{s.h, f_add(s.l, f_add(a.l, b.l))};
+}
+PF_FF_FN ff ff_sub_raw(ff a, ff b) { return ff_add_raw(a, ff_neg(b)); }
 // 1 + a
 PF_FF_FN ff ff_one_plus(ff a) { return ff_add(a, 1.0f); }
 
