@@ -12,8 +12,8 @@
 //     reciprocals of the FP64 path, an inexact correction is repaired by the next
 //     iteration's residual.  The one before the last takes its residual in ff
 //     (pf_ff.cuh, sums not renormalised), those before it in FP32.  (The Adams methods
-//     evaluate and solve in ff: their explicit predictors are far off on stiff
-//     particles, where an inexact first step would be seen in the K-th.)
+//     evaluate and solve in ff up to there: their explicit predictors are far off on
+//     stiff particles, where an inexact first step would be seen in the K-th.)
 //   - the last evaluates G in FP64 at the point y = x_n + (leading float of D).
 //     Its correction is D's low float, known, plus a rest of about 2^-50 |y| that an
 //     FP32 solution serves; what FP32 made of the point does not matter, since G
@@ -27,8 +27,8 @@
 //
 // A Robertson BDF2 substep with error sums takes 15 FP64 instructions instead
 // of 89, an M1 one 19 instead of 186.  Measured (GB300, device time):
-// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.234 ms, stage 2 1.08 -> 0.293 ms;
-// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.065 and 0.23 -> 0.077 ms (the exponentials and
+// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.231 ms, stage 2 1.08 -> 0.290 ms;
+// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.065 and 0.23 -> 0.075 ms (the exponentials and
 // roots of pf_math.cuh and the register bounds included).  Accuracy over an interval,
 // against quadruple precision on 200 particles of the prior, 2-norm of the state:
 // Robertson 3e-17 (plain FP64 9e-16), M1 6e-17 (4e-16).
@@ -206,9 +206,9 @@ struct RobertsonFast {
     const double q64 = T.k3 * y2;
     const double s64 = fma(T.k1, y1, -(q64 * y3));  // k1 y1 - k3 y2 y3 = -f1
     const double c64 = (T.k2 * y2) * y2;            // k2 y2^2 = f3
-    const ff G1 = ff_add(ff_from(fma(c.gamma, s64, st.R64[0])), st.cor[0]);
-    const ff G2 = ff_add(ff_from(fma(-c.gamma, s64, fma(c.gamma, c64, st.R64[1]))), st.cor[1]);
-    const ff G3 = ff_add(ff_from(fma(-c.gamma, c64, st.R64[2])), st.cor[2]);
+    const ff G1 = ff_add_raw(ff_from(fma(c.gamma, s64, st.R64[0])), st.cor[0]);
+    const ff G2 = ff_add_raw(ff_from(fma(-c.gamma, s64, fma(c.gamma, c64, st.R64[1]))), st.cor[1]);
+    const ff G3 = ff_add_raw(ff_from(fma(-c.gamma, c64, st.R64[2])), st.cor[2]);
     const float e1 = f_from(y1), e2f = f_from(y2), e3 = f_from(y3);
     // G + (I - gamma J) lo: what the low floats leave to correct
     const float q = f_mul(k.gk3.h, e2f), p = f_mul(k.gk3.h, e3), t = f_mul(k.gk2.h, e2f), w = f_add(t, t);
@@ -350,10 +350,10 @@ struct MichaelisFast {
     fy[0] = gk.f0 + w1;
     fy[1] = (k.vd - w1) + w2;
     fy[2] = fma(-kLambda, st.y[2], k.vc) - w2;
-    const ff gd1 = ff_mul(c.g, du1), gd2 = ff_mul(c.g, du2);
-    const ff G1 = ff_sub(ff_add(ff_from(fma(-c.gamma, fy[0], st.R64[0])), st.cor[0]), gd1);
-    const ff G2 = ff_sub(ff_add(ff_add(ff_from(fma(-c.gamma, fy[1], st.R64[1])), st.cor[1]), gd1), gd2);
-    const ff G3 = ff_add(ff_add(ff_from(fma(-c.gamma, fy[2], st.R64[2])), st.cor[2]), gd2);
+    const ff gd1 = ff_mul_raw(c.g, du1), gd2 = ff_mul_raw(c.g, du2);
+    const ff G1 = ff_sub_raw(ff_add_raw(ff_from(fma(-c.gamma, fy[0], st.R64[0])), st.cor[0]), gd1);
+    const ff G2 = ff_sub_raw(ff_add_raw(ff_add_raw(ff_from(fma(-c.gamma, fy[1], st.R64[1])), st.cor[1]), gd1), gd2);
+    const ff G3 = ff_add_raw(ff_add_raw(ff_from(fma(-c.gamma, fy[2], st.R64[2])), st.cor[2]), gd2);
     // G + (I - gamma J) lo: what the low floats leave to correct
     const float ga = f_mul(f_mul(c.g.h, u1), r1.h), gb = f_mul(f_mul(c.g.h, u2), r2.h);
     const float al = f_mul(ga, st.lo[0]), bl = f_mul(gb, st.lo[1]);
@@ -408,7 +408,7 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
   ff P[3], Dv[3], xf[3];
   FastState st;
   for (int i = 0; i < 3; ++i) {
-    xf[i] = ff_add(ff_from(w.x[i]), w.cx[i]);
+    xf[i] = ff_add_raw(ff_from(w.x[i]), w.cx[i]);
     if (!ERR && FAM != 2) {
       // a start for the iterations only: a float does
       float p = f_fma(c.pb.h, w.fb[i].h, f_fma(c.pa.h, w.fa[i].h, f_mul(c.ep, xf[i].h)));
@@ -430,7 +430,8 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
     }
     for (int it = 0; it + 1 < K; ++it) {
       if (FAM != 2 && it + 2 < K) MF::first(fk, gk, c, xf, R, Dv);
-      else MF::template early<FAM == 2>(fk, gk, c, xf, R, Dv);
+      else if (FAM == 2 && (it + 2 < K || K == 2)) MF::template early<true>(fk, gk, c, xf, R, Dv);
+      else MF::template early<false>(fk, gk, c, xf, R, Dv);
     }
   }
   float hh[3];
@@ -448,7 +449,7 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
     else r = ff_mul_raw(c.fra, w.ra[i]);
     if (FAM == 1) r = ff_fma(c.frb, w.rb[i], r);
     if (FAM != 2) r.l = f_fma(-c.er, xf[i].h, r.l);
-    st.cor[i] = ff_sub(r, w.cx[i]);
+    st.cor[i] = ff_sub_raw(r, w.cx[i]);
   }
   ff dl[3], dfy[3];
   double fy[3];
