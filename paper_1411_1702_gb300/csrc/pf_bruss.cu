@@ -19,10 +19,11 @@
 // an FP32 solution for the rest; where that rest is not small enough for FP32
 // to be exact beside the state, one step of refinement in ff follows.  A
 // particle the floats do not serve repeats the substep in FP64 on the same
-// lanes.  Measured (GB300, S = 20, stage 1 + stage 2): N = 1000 7.3 -> 0.22 ms,
-// N = 16384 8.57 -> 1.50 ms, N = 65536 23.4 -> 5.7 ms; the FP64 pipe is 60 %
+// lanes.  Measured (GB300, S = 20, stage 1 + stage 2): N = 1000 7.3 -> 0.21 ms,
+// N = 16384 8.57 -> 1.45 ms, N = 65536 23.4 -> 5.5 ms; the FP64 pipe is 60 %
 // busy, three warps a sub-partition (168 registers) waiting on each other's
-// results the rest; 128 registers (four warps, spills) and 64-thread blocks
+// results the rest (the launch bound keeps the three: at 177 registers stage 2 of N =
+// 16384 took 0.97 ms, at 168 0.79); 128 registers (four warps, spills) and 64-thread blocks
 // changed the epochs by less than 4 %.
 #include "pf_epoch.cuh"
 #include "pf_fast.cuh"
@@ -213,22 +214,24 @@ __device__ __forceinline__ void br_residual32(const BrPar& T, const BrDiag<float
   }
 }
 
-// the same with G in ff
+// the same with G in ff, sums not renormalised
 __device__ __forceinline__ void br_residual_ff(const BrPar& T, const BrDiag<float>& c, ff gf, const ff (&x)[4],
                                                const ff (&Rv)[4], const ff (&Dv)[4], int g, float (&mG)[4],
                                                Mat2<float> (&M)[2]) {
   ff y[4], L[4], R[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) y[k] = ff_add(x[k], Dv[k]);
+  for (int k = 0; k < 4; ++k) y[k] = ff_add_raw(x[k], Dv[k]);
   br_neighbours(y, g, ff{1.0f, 0.0f}, ff{3.0f, 0.0f}, L, R);
 #pragma unroll
   for (int k = 0; k < 4; k += 2) {
-    const ff u = y[k], v = y[k + 1], uuv = ff_mul(ff_mul(u, u), v);
-    const ff lu = ff_sub(ff_add(L[k], R[k]), ff_twice(u)), lv = ff_sub(ff_add(L[k + 1], R[k + 1]), ff_twice(v));
-    const ff fu = ff_fma(T.D, lu, ff_sub(ff_add(T.A, uuv), ff_mul(T.B1, u)));
-    const ff fv = ff_fma(T.D, lv, ff_sub(ff_mul(T.B, u), uuv));
-    mG[k] = ff_sub(ff_mul(gf, fu), ff_add(Dv[k], Rv[k])).h;
-    mG[k + 1] = ff_sub(ff_mul(gf, fv), ff_add(Dv[k + 1], Rv[k + 1])).h;
+    const ff u = y[k], v = y[k + 1], uuv = ff_mul_raw(ff_mul_raw(u, u), v);
+    const ff lu = ff_sub_raw(ff_add_raw(L[k], R[k]), ff_twice(u)), lv = ff_sub_raw(ff_add_raw(L[k + 1], R[k + 1]), ff_twice(v));
+    const ff fu = ff_add_raw(ff_mul_raw(T.D, lu), ff_sub_raw(ff_add_raw(T.A, uuv), ff_mul_raw(T.B1, u)));
+    const ff fv = ff_add_raw(ff_mul_raw(T.D, lv), ff_sub_raw(ff_mul_raw(T.B, u), uuv));
+    const ff mu = ff_sub_raw(ff_mul_raw(gf, fu), ff_add_raw(Dv[k], Rv[k]));
+    const ff mv = ff_sub_raw(ff_mul_raw(gf, fv), ff_add_raw(Dv[k + 1], Rv[k + 1]));
+    mG[k] = f_add(mu.h, mu.l);
+    mG[k + 1] = f_add(mv.h, mv.l);
     M[k / 2] = br_block(c, u.h, v.h);
   }
 }
@@ -571,7 +574,7 @@ __device__ __forceinline__ void bstage2_body(const FilterDev& fd, const EpochPar
 }
 
 template <int STAGE>
-__global__ void __launch_bounds__(kBrThreads) k_bstage(const __grid_constant__ FilterDev fd,
+__global__ void __launch_bounds__(kBrThreads, 3) k_bstage(const __grid_constant__ FilterDev fd,
                                                      const EpochParams* __restrict__ ep) {
   extern __shared__ double s_dyn[];
   __shared__ double s_red[32];
@@ -584,7 +587,7 @@ __global__ void __launch_bounds__(kBrThreads) k_bstage(const __grid_constant__ F
 }
 
 template <int STAGE>
-__global__ void __launch_bounds__(kBrThreads) k_batch_bstage(const FilterDev* __restrict__ fds,
+__global__ void __launch_bounds__(kBrThreads, 3) k_batch_bstage(const FilterDev* __restrict__ fds,
                                                            const EpochParams* const* __restrict__ eps,
                                                            const BatchTile* __restrict__ tiles) {
   extern __shared__ double s_dyn[];
