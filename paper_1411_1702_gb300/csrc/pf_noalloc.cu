@@ -109,18 +109,17 @@ __global__ void __launch_bounds__(256) k_na_scan_add(int64_t N, int items, doubl
 }
 
 // the filter's merge-path search (resample_tile), one block per diagonal tile;
-// corners: found first by k_na_corners (two-phase), or null
-__global__ void __launch_bounds__(kResampleThreads, 4) k_na_resample(const double* __restrict__ c,
-                                                                  int64_t N, double u,
-                                                                  int32_t* __restrict__ idx,
-                                                                  const int32_t* __restrict__ corners) {
+// corners: found first by k_na_corners (two-phase), or null.  (c and corners are
+// written by kernels this one is launched beside: not __restrict__, see CumFinal.)
+__global__ void __launch_bounds__(kResampleThreads, 4) k_na_resample(const double* c, int64_t N, double u,
+                                                                  int32_t* idx, const int32_t* corners) {
   __shared__ RsShared sh;
   pdl_wait();
   resample_tile(CumFinal{c}, N, u, idx, nullptr, blockIdx.x, sh, corners);
 }
 
-__global__ void __launch_bounds__(256) k_na_corners(const double* __restrict__ c, int64_t N, double u,
-                                                   int32_t* __restrict__ corners) {
+__global__ void __launch_bounds__(256) k_na_corners(const double* c, int64_t N, double u,
+                                                   int32_t* corners) {
   pdl_wait();
   pdl_trigger();
   rs_corners_core(CumFinal{c}, N, u, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, corners);

@@ -227,9 +227,14 @@ __device__ __forceinline__ void scan_add_core(const ScanArgs& a, int64_t k) {
 // sums) read through the per-tile offsets and floors, c_k = max(boff_t + cl_k,
 // pmax_t) for the tile t holding k: the offset pass (scan_add_core) folded
 // into the reads, bit for bit the values it would store.
+// Their kernels are launched with programmatic dependence, so the kernels that
+// write these arrays are still running when they start: the reads are ordinary
+// loads after pdl_wait(), which orders them.  (Loads of the read-only path, __ldg
+// or through a const __restrict__ kernel argument, are for data that nothing
+// writes while the kernel runs; the wait does not order those.)
 struct CumFinal {
   const double* c;
-  __device__ __forceinline__ double operator()(int64_t k) const { return __ldg(c + k); }
+  __device__ __forceinline__ double operator()(int64_t k) const { return c[k]; }
 };
 
 struct CumTiles {
@@ -239,7 +244,7 @@ struct CumTiles {
   uint32_t len;  // tile length, scan_tile_len(N, sms)
   __device__ __forceinline__ double operator()(int64_t k) const {
     const uint32_t t = (uint32_t)k / len;
-    return max_nonneg(__ldg(boff + t) + __ldg(cl + k), __ldg(pmax + t));
+    return max_nonneg(boff[t] + cl[k], pmax[t]);
   }
 };
 
@@ -348,7 +353,7 @@ __host__ __device__ inline unsigned rs_corner_blocks(int64_t N) {
 // Every lane of the warp calls it with the same v.
 template <class V>
 __device__ __forceinline__ void rs_corners_core(const V& c, int64_t N, double u, int64_t v,
-                                                int32_t* __restrict__ corners) {
+                                                int32_t* corners) {
   if (v > rs_tiles(N)) return;
   RsTau t;
   t.u = u;
@@ -369,7 +374,7 @@ template <class V>
 __device__ __forceinline__ void resample_tile(const V& c, int64_t N, double u,
                                               int32_t* __restrict__ idx,
                                               unsigned long long* n_unique, int vb, RsShared& sh,
-                                              const int32_t* __restrict__ corners = nullptr) {
+                                              const int32_t* corners = nullptr) {
   // the block's tile of the merge: items [d0, d1), taus [a0, a1), c [b0, b1)
   const int64_t d0 = (int64_t)vb * kRsTile;
   const int64_t d1 = d0 + kRsTile < 2 * N ? d0 + kRsTile : 2 * N;
@@ -382,7 +387,7 @@ __device__ __forceinline__ void resample_tile(const V& c, int64_t N, double u,
     t.step = t.total / (double)N;
     t.ustep = u * t.step;
     // the corners: given (two-phase), else a warp-wide search each
-    const int64_t a = corners ? (int64_t)__ldg(corners + vb + wid) : rs_corner(c, wid == 0 ? d0 : d1, t);
+    const int64_t a = corners ? (int64_t)corners[vb + wid] : rs_corner(c, wid == 0 ? d0 : d1, t);
     if (lane == 0) {
       sh.corner[wid] = a;
       if (wid == 0) {
