@@ -383,8 +383,9 @@ constexpr int kAdNaN = 1 << 20;
 __device__ __forceinline__ double ad_unit(int k) {
   return k == kAdNaN ? CUDART_NAN : d_from((uint32_t)(k + 1023) << 20, 0u);
 }
+// (0 below the floats' normal range)
 __device__ __forceinline__ float ad_unit_f(int k) {
-  return k >= kAdNaN / 2 ? CUDART_NAN_F : f_from_bits((uint32_t)(k + 127) << 23);
+  return k > 127 ? CUDART_NAN_F : k < -126 ? 0.0f : f_from_bits((uint32_t)(k + 127) << 23);
 }
 
 // Inverse: the threads' modes z give, per particle q,
@@ -584,6 +585,11 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
   __shared__ double s_th[PB][kPMax];
   __shared__ unsigned s_top[3][2 * PB];  // scales of the fields, then of successive inverses
   __shared__ unsigned s_state[PB];    // the largest high word of the state's modes
+  // Scale 2^s_err of the estimates squared and summed in ff: 2^40 over the size 2^e of
+  // the state's modes, so that it follows the state's units.  An estimate up to 2^(e +
+  // 18) squares and sums within the floats; one that may be above (V 2^k, |V| < 2^62: k +
+  // 62 > e + 18) is summed in FP64.
+  __shared__ int s_err[PB];
   __shared__ int s_flag;
   const Ctrl* ctrl = fd.ctrl;
   if (ctrl->status != PF_OK) return;
@@ -710,6 +716,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
     }
   }
   __syncthreads();
+  if (STAGE == 2 && tid < PB) s_err[tid] = 40 - fx_scale(s_state[tid]);  // (read after the first inverse's barriers)
   double lr[U][2], li[U][2];
 #pragma unroll
   for (int j = 0; j < U; ++j) {
@@ -833,11 +840,18 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
         }
       } else {
         ad_inverse(L, sm, top, e, [&](int q, int i, long long V, int k) {
-          ff* EE = reinterpret_cast<ff*>(sm + L.base + q * L.per + L.F[2]);
-          ff v = ff_from((double)V);
-          const float u = ad_unit_f(k + 40);  // times kErrScale
-          v = ff{f_mul(v.h, u), f_mul(v.l, u)};
-          EE[i] = ff_fma(v, v, EE[i]);
+          double* R = sm + L.base + q * L.per;
+          const int ku = k + s_err[q];
+          if (ku <= -4) {
+            ff* EE = reinterpret_cast<ff*>(R + L.F[2]);
+            ff v = ff_from((double)V);
+            const float u = ad_unit_f(ku);
+            v = ff{f_mul(v.h, u), f_mul(v.l, u)};
+            EE[i] = ff_fma(v, v, EE[i]);
+          } else {  // (also one that is not finite)
+            const double v = (double)V * ad_unit(k);
+            R[L.F[1] + i] = fma(v, v, R[L.F[1] + i]);
+          }
         });
       }
     }
@@ -871,7 +885,8 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
       for (int h = 0; h < 2; ++h) {
         const int i = 2 * b + h;
         if (i >= d) break;
-        const double E = fma(value_of(reinterpret_cast<ff*>(R + L.F[2])[i]), kErrUnscale, R[L.F[1] + i]);
+        const double u = ad_unit(-s_err[q]);
+        const double E = fma(value_of(reinterpret_cast<ff*>(R + L.F[2])[i]) * u, u, R[L.F[1] + i]);
         R[L.F[2] + i] = pfm::sqrt_fixed(fd.kappa * E) * (h == 0 ? z0 : z1);
       }
     }
