@@ -608,31 +608,31 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
   const int d = L.d, nt = L.nt, H = L.H, T = blockDim.x, tid = threadIdx.x, units = H * H;
   const double inv_d = 1.0 / (double)d;
   // particle q of the block is n0 + q, gathered from slot l (stage 2: the
-  // resampled parent); slots past N are idle and stay zero
-  auto slot_of = [&](int q) -> int64_t { return STAGE == 2 ? (int64_t)fd.idx[n0 + q] : n0 + q; };
+  // resampled parent); slots past N repeat the last particle and write nothing, so
+  // that they have no say in when the block's estimates leave FP64
+  auto particle = [&](int q) -> int64_t { return n0 + q < N ? n0 + q : N - 1; };
+  auto slot_of = [&](int q) -> int64_t { return STAGE == 2 ? (int64_t)fd.idx[particle(q)] : particle(q); };
   if (tid < PB) {
     const int q = tid;
-    const int64_t n = n0 + q;
-    double ph[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    if (n < N) {
-      const int64_t l = slot_of(q);
-      if (STAGE == 1) {
-        // Step 2: phibar^n = a phi^n + (1 - a) phibar
-        for (int i = 0; i < 5; ++i) ph[i] = fd.a * src.phi[i * N + n] + (1.0 - fd.a) * ctrl->phibar[i];
-      } else {
-        // Step 4a: phi_{j+1}^n = phibar^l + s L z
-        double z[6];
-        for (int b = 0; b < 3; ++b) {
-          const U4 w = draw_block(fd, kRngTheta, (uint32_t)n, epoch, (uint32_t)b);
-          normal_pair(w, z[2 * b], z[2 * b + 1]);
-        }
-        for (int i = 0; i < 5; ++i) {
-          double lz = 0.0;
-          for (int k = 0; k <= i; ++k) lz = fma(ctrl->L[i * kPMax + k], z[k], lz);
-          const double shr = fd.a * src.phi[i * N + l] + (1.0 - fd.a) * ctrl->phibar[i];
-          ph[i] = fma(fd.s, lz, shr);
-          dst.phi[i * N + n] = ph[i];
-        }
+    const int64_t n = particle(q);
+    double ph[5];
+    const int64_t l = slot_of(q);
+    if (STAGE == 1) {
+      // Step 2: phibar^n = a phi^n + (1 - a) phibar
+      for (int i = 0; i < 5; ++i) ph[i] = fd.a * src.phi[i * N + n] + (1.0 - fd.a) * ctrl->phibar[i];
+    } else {
+      // Step 4a: phi_{j+1}^n = phibar^l + s L z
+      double z[6];
+      for (int b = 0; b < 3; ++b) {
+        const U4 w = draw_block(fd, kRngTheta, (uint32_t)n, epoch, (uint32_t)b);
+        normal_pair(w, z[2 * b], z[2 * b + 1]);
+      }
+      for (int i = 0; i < 5; ++i) {
+        double lz = 0.0;
+        for (int k = 0; k <= i; ++k) lz = fma(ctrl->L[i * kPMax + k], z[k], lz);
+        const double shr = fd.a * src.phi[i * N + l] + (1.0 - fd.a) * ctrl->phibar[i];
+        ph[i] = fma(fd.s, lz, shr);
+        if (n0 + q < N) dst.phi[i * N + n] = ph[i];
       }
     }
     for (int i = 0; i < 5; ++i) s_th[q][i] = (fd.transform == PF_TRANSFORM_LOG) ? pfm::exp_fixed(ph[i]) : ph[i];
@@ -644,7 +644,6 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
   // scales of D1 and D2 (the error predictor's, stage 2)
   for (int t = tid; t < PB * d; t += T) {
     const int q = t / d;
-    if (n0 + q >= N) continue;
     const int64_t o = (int64_t)(t - q * d) * N + slot_of(q);
     const double x = src.x[o], h1 = src.h1[o];
     atomicMax(&s_top[1][q], hi_abs(x - h1));
@@ -658,17 +657,15 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 
     double* R = sm + L.base + q * L.per;
     const int my = py ? nt - py : 0, mxx = px ? nt - px : 0;
     const int at[4] = {py * nt + px, py * nt + mxx, my * nt + px, my * nt + mxx};
-    double x[4] = {0.0, 0.0, 0.0, 0.0}, e[4] = {0.0, 0.0, 0.0, 0.0}, f[4] = {0.0, 0.0, 0.0, 0.0};
-    if (n0 + q < N) {
-      const int64_t l = slot_of(q);
+    double x[4], e[4], f[4];
+    const int64_t l = slot_of(q);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int64_t o = (int64_t)at[i] * N + l;
-        x[i] = src.x[o];
-        const double h1 = src.h1[o];
-        e[i] = x[i] - h1;
-        if (STAGE == 2) f[i] = h1 - src.h2[o];
-      }
+    for (int i = 0; i < 4; ++i) {
+      const int64_t o = (int64_t)at[i] * N + l;
+      x[i] = src.x[o];
+      const double h1 = src.h1[o];
+      e[i] = x[i] - h1;
+      if (STAGE == 2) f[i] = h1 - src.h2[o];
     }
     const bool y0 = py == 0, x0 = px == 0;
     ad_fold(R + L.F[0], units, v, y0, x0, x[0], x[1], x[2], x[3]);
