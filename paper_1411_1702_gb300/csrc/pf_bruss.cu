@@ -264,10 +264,18 @@ struct BrCarry {
   ff fa[4], fb[4], E[4];
 };
 
+// What substeps in FP64 add in doubles, for values beyond the floats: their part of the
+// error sums and, while `b64` says so, b.  In shared memory, a column a thread:
+// registers are short, and few particles use it.
+struct BrWide {
+  double E[4][kBrThreads], b[4][kBrThreads];
+};
+
 // One substep in FP64, on all lanes of the warp: K Newton iterations in
 // increments from the same start.
 template <bool ERR>
-__device__ __noinline__ void br_step_fp64(const BrTheta& T, const StepCoef& c, int K, int g, BrCarry& w) {
+__device__ __noinline__ void br_step_fp64(const BrTheta& T, const StepCoef& c, int K, int g, BrCarry& w, BrWide* wide,
+                                          bool b64, bool mine) {
   double D0[4], P[4], R[4], xn[4], h1[4];
   double f[4];
   br_f(T, w.x, g, f);
@@ -275,7 +283,7 @@ __device__ __noinline__ void br_step_fp64(const BrTheta& T, const StepCoef& c, i
   for (int k = 0; k < 4; ++k) {
     xn[k] = w.x[k];
     h1[k] = w.x[k] - w.a[k];
-    const double h2 = h1[k] - ((double)w.fb[k].h + (double)w.fb[k].l);
+    const double h2 = h1[k] - (b64 ? wide->b[k][threadIdx.x] : (double)w.fb[k].h + (double)w.fb[k].l);
     // the start and the error predictor as increments
     D0[k] = c.kind == 2 ? fma(c.pi2, h2, fma(c.pi1, h1[k], c.pi0 * xn[k])) - xn[k] : 0.0;
     P[k] = c.kind == 2 ? D0[k] : c.h * f[k];
@@ -299,9 +307,10 @@ __device__ __noinline__ void br_step_fp64(const BrTheta& T, const StepCoef& c, i
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const double xk = xn[k] + D0[k];
-    if (ERR) {
-      const double e = c.mu * kErrScale * (D0[k] - P[k]);
-      w.E[k] = ff_add(w.E[k], ff_from(e * e));
+    if (mine) {
+      wide->b[k][threadIdx.x] = w.a[k];
+      const double e = c.mu * (D0[k] - P[k]);
+      if (ERR) wide->E[k][threadIdx.x] = fma(e, e, wide->E[k][threadIdx.x]);
     }
     w.a[k] = xk - xn[k];
     w.fb[k] = w.fa[k];
@@ -382,7 +391,14 @@ __device__ __forceinline__ unsigned br_step(const BrTheta& T, const BrPar& par, 
   }
   // finite, and the iterations settled (a single one: 2^-40 of it, after two FP32 solves,
   // below the last bit)
-  const bool ok = !far && md <= (K > 1 ? 0x1.0p-20f : 0x1.0p-13f) * my && my < 0x1.0p60f;
+  bool ok = !far && md <= (K > 1 ? 0x1.0p-20f : 0x1.0p-13f) * my && my < 0x1.0p60f;
+  if (ERR) {
+    // and squares of the scaled estimates whose sum stays a float (640 of 2^116)
+    float me = md;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) me = f_add(me, f_add(fabsf(P[k].h), fabsf(Dv[k].h)));
+    ok = ok && f_mul(fabsf(c.mus.h), me) < 0x1.0p58f;
+  }
   const unsigned bad = __ballot_sync(0xffffffffu, !ok);
   if (bad & ((threadIdx.x & 16u) ? 0xffff0000u : 0x0000ffffu)) return bad;
 #pragma unroll
@@ -403,10 +419,10 @@ __device__ __forceinline__ unsigned br_step(const BrTheta& T, const BrPar& par, 
   return bad;
 }
 
-// Psi over the S substeps for the warp's two particles.
+// Psi over the S substeps for the warp's two particles; returns whether wide->b holds b.
 template <bool ERR>
-__device__ __forceinline__ void br_propagate(const StepCoef* sc, const FastCoef* fc, int S, int K, const BrTheta& T,
-                                             int g, BrCarry& w) {
+__device__ __forceinline__ bool br_propagate(const StepCoef* sc, const FastCoef* fc, int S, int K, const BrTheta& T,
+                                             int g, BrCarry& w, BrWide* wide) {
   const BrPar par{ff_from(T.A), ff_from(T.B), ff_from(T.B + 1.0), ff_from(T.D)};
   const unsigned group = (threadIdx.x & 16u) ? 0xffff0000u : 0x0000ffffu;
   // the range in which the floats serve
@@ -414,7 +430,12 @@ __device__ __forceinline__ void br_propagate(const StepCoef* sc, const FastCoef*
 #pragma unroll
   for (int k = 0; k < 4; ++k) big = fmax(big, fabs(w.x[k]));
   const double tb = fmax(fmax(fabs(T.A), fabs(T.B)), fabs(T.D));
-  const bool far = !(big <= kFastStateMax && tb <= kFastThetaMax);
+  // (a particle with a component that is not far below the floats' 1)
+  float top = f_from(big);
+#pragma unroll
+  for (int o = 1; o < kBrLanes; o *= 2) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+  const bool far = !(big <= kFastStateMax && tb <= kFastThetaMax && top >= (float)kFastStateMin);
+  bool b64 = true;
 #pragma unroll 1
   for (int s = 0; s < S; ++s) {
     const FastCoef& c = fc[s];
@@ -423,14 +444,16 @@ __device__ __forceinline__ void br_propagate(const StepCoef* sc, const FastCoef*
     if (bad) {
       // on a copy, so that the carry itself stays in registers
       BrCarry t = w;
-      br_step_fp64<ERR>(T, sc[s], K, g, t);
+      br_step_fp64<ERR>(T, sc[s], K, g, t, wide, b64, (bad & group) != 0);
       if (bad & group) w = t;
     }
+    b64 = (bad & group) != 0;
   }
+  return b64;
 }
 
 // The lane's four components of a particle's history from SoA rows.
-__device__ __forceinline__ void br_load(const Ensemble& E, int64_t N, int64_t l, int g, BrCarry& w) {
+__device__ __forceinline__ void br_load(const Ensemble& E, int64_t N, int64_t l, int g, BrCarry& w, BrWide* wide) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int64_t o = (int64_t)(4 * g + k) * N + l;
@@ -438,7 +461,10 @@ __device__ __forceinline__ void br_load(const Ensemble& E, int64_t N, int64_t l,
     w.x[k] = x;
     w.a[k] = x - h1;
     w.fa[k] = ff_from(w.a[k]);
-    w.fb[k] = ff_from(h1 - h2);
+    const double b = h1 - h2;
+    w.fb[k] = ff_from(b);
+    wide->b[k][threadIdx.x] = b;
+    wide->E[k][threadIdx.x] = 0.0;
     w.cx[k] = w.ca[k] = 0.0f;
     w.E[k] = ff{0.0f, 0.0f};
   }
@@ -469,7 +495,7 @@ __device__ __forceinline__ const FastCoef* br_tables(StepCoef* s_sc, const Epoch
 
 __device__ __forceinline__ void bstage1_body(const FilterDev& fd, const EpochParams* __restrict__ ep,
                                              int vb, int vg, const StepCoef* s_sc, const FastCoef* s_fc,
-                                             double* s_red, int* s_flag) {
+                                             BrWide* wide, double* s_red, int* s_flag) {
   const Ctrl* ctrl = fd.ctrl;
   const Ensemble src = committed(fd, ctrl->cur);
   const int64_t N = fd.N;
@@ -481,8 +507,8 @@ __device__ __forceinline__ void bstage1_body(const FilterDev& fd, const EpochPar
   for (int i = 0; i < 3; ++i) ph[i] = fd.a * src.phi[i * N + n] + (1.0 - fd.a) * ctrl->phibar[i];
   to_theta<3>(fd, ph, th);
   BrCarry w;
-  br_load(src, N, n, g, w);
-  br_propagate<false>(s_sc, s_fc, ep->S, fd.K, br_theta(th), g, w);
+  br_load(src, N, n, g, w, wide);
+  br_propagate<false>(s_sc, s_fc, ep->S, fd.K, br_theta(th), g, w, wide);
   double x[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) x[k] = w.x[k] + (double)w.cx[k];
@@ -499,7 +525,7 @@ __device__ __forceinline__ void bstage1_body(const FilterDev& fd, const EpochPar
 
 __device__ __forceinline__ void bstage2_body(const FilterDev& fd, const EpochParams* __restrict__ ep,
                                              int vb, int vg, const StepCoef* s_sc, const FastCoef* s_fc,
-                                             double* s_red, int* s_flag) {
+                                             BrWide* wide, double* s_red, int* s_flag) {
   const Ctrl* ctrl = fd.ctrl;
   const int cur = ctrl->cur;
   const Ensemble src = committed(fd, cur);
@@ -530,9 +556,9 @@ __device__ __forceinline__ void bstage2_body(const FilterDev& fd, const EpochPar
   }
   to_theta<3>(fd, ph, th);
   BrCarry w;
-  br_load(src, N, l, g, w);
+  br_load(src, N, l, g, w, wide);
   // 4b, 4d: repropagate with the Milne error sums
-  br_propagate<true>(s_sc, s_fc, ep->S, fd.K, br_theta(th), g, w);
+  const bool b64 = br_propagate<true>(s_sc, s_fc, ep->S, fd.K, br_theta(th), g, w, wide);
   // 4c, 4d: innovation
   double x[4];
 #pragma unroll
@@ -544,11 +570,11 @@ __device__ __forceinline__ void bstage2_body(const FilterDev& fd, const EpochPar
     for (int h = 0; h < 2; ++h) {
       const int k = 2 * b + h;
       const int64_t o = (int64_t)(4 * g + k) * N + n;
-      const double E = ((double)w.E[k].h + (double)w.E[k].l) * kErrUnscale;
+      const double E = fma((double)w.E[k].h + (double)w.E[k].l, kErrUnscale, wide->E[k][threadIdx.x]);
       const double v = pfm::sqrt_fixed(fd.kappa * E) * (h == 0 ? z0 : z1);
       const double xk = w.x[k] + (double)w.cx[k];
       const double h1 = xk - (w.a[k] + (double)w.ca[k]);
-      const double h2 = h1 - ((double)w.fb[k].h + (double)w.fb[k].l);
+      const double h2 = h1 - (b64 ? wide->b[k][threadIdx.x] : (double)w.fb[k].h + (double)w.fb[k].l);
       x[k] = xk + v;
       if (live) {
         dst.x[o] = x[k];
@@ -578,12 +604,13 @@ __global__ void __launch_bounds__(kBrThreads, 3) k_bstage(const __grid_constant_
                                                      const EpochParams* __restrict__ ep) {
   extern __shared__ double s_dyn[];
   __shared__ double s_red[32];
+  __shared__ BrWide s_wide;
   __shared__ int s_flag;
   if (fd.ctrl->status != PF_OK) return;
   StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
   const FastCoef* s_fc = br_tables(s_sc, ep, ep->S);
-  if (STAGE == 1) bstage1_body(fd, ep, blockIdx.x, gridDim.x, s_sc, s_fc, s_red, &s_flag);
-  else bstage2_body(fd, ep, blockIdx.x, gridDim.x, s_sc, s_fc, s_red, &s_flag);
+  if (STAGE == 1) bstage1_body(fd, ep, blockIdx.x, gridDim.x, s_sc, s_fc, &s_wide, s_red, &s_flag);
+  else bstage2_body(fd, ep, blockIdx.x, gridDim.x, s_sc, s_fc, &s_wide, s_red, &s_flag);
 }
 
 template <int STAGE>
@@ -592,6 +619,7 @@ __global__ void __launch_bounds__(kBrThreads, 3) k_batch_bstage(const FilterDev*
                                                            const BatchTile* __restrict__ tiles) {
   extern __shared__ double s_dyn[];
   __shared__ double s_red[32];
+  __shared__ BrWide s_wide;
   __shared__ int s_flag;
   const BatchTile t = tiles[blockIdx.x];
   const FilterDev& fd = *(fds + t.f);
@@ -600,8 +628,8 @@ __global__ void __launch_bounds__(kBrThreads, 3) k_batch_bstage(const FilterDev*
   StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
   const FastCoef* s_fc = br_tables(s_sc, ep, ep->S);
   const int vg = (int)((fd.N + kBrPerBlock - 1) / kBrPerBlock);
-  if (STAGE == 1) bstage1_body(fd, ep, t.vb, vg, s_sc, s_fc, s_red, &s_flag);
-  else bstage2_body(fd, ep, t.vb, vg, s_sc, s_fc, s_red, &s_flag);
+  if (STAGE == 1) bstage1_body(fd, ep, t.vb, vg, s_sc, s_fc, &s_wide, s_red, &s_flag);
+  else bstage2_body(fd, ep, t.vb, vg, s_sc, s_fc, &s_wide, s_red, &s_flag);
 }
 
 int bruss_stage_blocks(int64_t N) { return (int)((N + kBrPerBlock - 1) / kBrPerBlock); }
