@@ -376,12 +376,17 @@ __device__ __forceinline__ unsigned br_step(const BrTheta& T, const BrPar& par, 
     dl[k] = two_sum(lo[k], d[k]);
   }
   // FP32 solutions are good to about 2^-20: beside y that is exact for a
-  // correction of 2^-34 |y|, else the defect is solved for once more
-  if (__any_sync(0xffffffffu, !(md <= 0x1.0p-34f * my))) {
+  // correction of 2^-34 |y|, else the defect is solved for once more (by the warp, for
+  // those of its two particles that need it: a particle's result is its own)
+  const unsigned group = (threadIdx.x & 16u) ? 0xffff0000u : 0x0000ffffu;
+  const unsigned refine = __ballot_sync(0xffffffffu, !(md <= 0x1.0p-34f * my));
+  if (refine) {
     br_defect(par, c.g, y, G, dl, g, mG);
     br_solve(M, q.gD, g, mG, d);
+    if (refine & group) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) dl[k] = ff_add(dl[k], d[k]);
+      for (int k = 0; k < 4; ++k) dl[k] = ff_add(dl[k], d[k]);
+    }
   }
   if (ERR && kind != 2) {
     // a cold start's error predictor is the explicit-Euler step
@@ -400,7 +405,7 @@ __device__ __forceinline__ unsigned br_step(const BrTheta& T, const BrPar& par, 
     ok = ok && f_mul(fabsf(c.mus.h), me) < 0x1.0p58f;
   }
   const unsigned bad = __ballot_sync(0xffffffffu, !ok);
-  if (bad & ((threadIdx.x & 16u) ? 0xffff0000u : 0x0000ffffu)) return bad;
+  if (bad & group) return bad;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const double xn = y[k] + d_from_f(dl[k].h);
