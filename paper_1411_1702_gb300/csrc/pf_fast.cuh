@@ -460,6 +460,11 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
   const float my = fabsf(f_from(st.y[0])) + fabsf(f_from(st.y[1])) + fabsf(f_from(st.y[2]));
   const float md = fabsf(dl[0].h) + fabsf(dl[1].h) + fabsf(dl[2].h);
   if (!(md <= (K > 1 ? MF::kSettled : kFastSingle) * my && my < 0x1.0p60f)) return false;
+  if (ERR) {
+    // and squares of the scaled estimates whose sum stays a float (640 of 2^116)
+    const float me = fabsf(P[0].h) + fabsf(P[1].h) + fabsf(P[2].h) + fabsf(hh[0]) + fabsf(hh[1]) + fabsf(hh[2]) + md;
+    if (!(fabsf(c.mus.h) * me < 0x1.0p58f)) return false;
+  }
   for (int i = 0; i < 3; ++i) {
     // the increment from x_n to the new state
     const ff rest = ff_sub(dl[i], w.cx[i]);

@@ -1,7 +1,8 @@
 """Error sums of the substeps (Step 4b) where the squared estimates leave the range of
 floats: the Brusselator with a source that makes its states large, on the FP64 path
-(parameters above 2^40) and before it, beyond the floats' own range, and tiny.
-Against the CPU oracle within the repository's bounds."""
+(parameters above 2^40) and before it, beyond the floats' own range, and tiny; and
+Robertson with a history far from its state.  Against the CPU oracle within the
+repository's bounds."""
 import numpy as np
 import pytest
 
@@ -40,5 +41,26 @@ def test_brusselator_sources(pf, A, u0):
     o.init()
     for k in range(3):
         check_epoch(g, o, w.t_obs[k], w.y_obs[k])
+    assert np.isfinite(g.pf_get_ensemble()["lw"]).all()
+    g.close()
+
+
+@pytest.mark.parametrize("jump", [2.0 ** 10, 2.0 ** 29])
+@pytest.mark.parametrize("lmm", [W.LMM_BDF2, W.LMM_BDF3])
+def test_robertson_far_history(pf, lmm, jump):
+    """A past `jump` away from the state, in a regime where the reactions are slow."""
+    w = W.robertson(N=33, T=3)
+    w = w.with_(lmm=lmm, spacing=W.SPACING_UNIFORM, dt=0.1, t_obs=np.array([1.0, 2.0, 3.0]), noise=W.NOISE_ADDITIVE,
+                sigma=[jump, jump], prior_lo=[0.02, 2.0 ** -39, 2.0 ** -39], prior_hi=[0.08, 2.0 ** -38, 2.0 ** -38],
+                x0=np.array([2.0 ** 9, 1.0, 1.0]))
+    y = np.array([[2.0 ** 9, 1.0]] * 3)
+    g, o = pf.Filter.from_workload(w), oracle.Filter(w)
+    o.init()
+    check_epoch(g, o, w.t_obs[0], y[0])
+    e = g.pf_get_ensemble()
+    h1 = e["h1"].copy()
+    h1[:, 0] += jump
+    g.pf_set_ensemble(h1=h1)
+    check_epoch(g, o, w.t_obs[1], y[1])
     assert np.isfinite(g.pf_get_ensemble()["lw"]).all()
     g.close()
