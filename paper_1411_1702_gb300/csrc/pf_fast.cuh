@@ -22,7 +22,7 @@
 // correction in ff, so a substep rounds it once, and Milne's estimate comes from
 // D - P without the cancellation of y - x_p.  The result is the K-th Newton
 // iterate to FP64 rounding, as before; a substep that does not satisfy this
-// reasoning (a non-finite value, a last correction that is not small, an
+// reasoning (a non-finite value, iterations that have not settled, an
 // exponent outside the floats') is left to the FP64 path by fast_run's caller.
 //
 // A Robertson BDF2 substep with error sums takes 15 FP64 instructions instead
@@ -46,13 +46,20 @@ constexpr double kErrScale = 0x1.0p40, kErrUnscale = 0x1.0p-80;
 constexpr double kFastStateMin = 0x1.0p-40, kFastStateMax = 0x1.0p20;
 constexpr double kFastThetaMin = 0x1.0p-40, kFastThetaMax = 0x1.0p40;
 constexpr float kFastStepMin = 0x1.0p-60f, kFastStepMax = 0x1.0p40f;
-// the largest correction beside the state of a single iteration (its ff solve is good
-// to 2^-46); of the last of several: the models' kSettled
-constexpr float kFastSingle = 0x1.0p-7f;
-// The last correction is D's low floats lo, known, and a rest: an FP32 solution, good to
-// 2^-20, serves a rest of up to 2^-34 of the state.  It is below 2^-44 for 99.5 % of the
-// substeps of the prior (K = 2 and 4).
-constexpr float kFastRest = 0x1.0p-34f;
+// The last correction is D's low floats lo, known, and a rest.  Both limits hold for each
+// component beside its own size (Robertson's y2 and y3 can be 1e-9 of y1).
+//  - An FP32 solution, good to 2^-20, serves a rest of up to 2^-32; above it the rest is
+//    solved for in ff (0.3 % of Robertson's substeps over its prior at S = 50, K = 2).
+//  - The point is off the (K-1)-th iterate by D's rounding to a float, and that by the
+//    early FP32 solves' 2^-22 of their step; the last iteration leaves both times the
+//    rest.  Above 2^-17 the substep is taken with all of that in ff and FP64 (WIDE): a few
+//    at the start of intervals whose parameters have just moved (stage 2: up to half a
+//    dozen of 50), and every one of K = 1.  The models' kSettled is what the rest may be
+//    then; a substep above it goes to FP64.  Over Robertson's prior, parameters moved by a
+//    fifth, y2 and y3 are within 5e-16 (S = 50, K = 2; FP64 path 3e-15) and 7e-15 (S = 2; 2e-10);
+//    limits of 2^-19 to 2^-26 give the same at S = 50.  With limits on the norm and no second
+//    form it was 1e-13 and 2e-10, and up to 6e-9 for K = 1.
+constexpr float kFastRest = 0x1.0p-32f, kFastSettled = 0x1.0p-17f;
 
 // One substep's coefficients for the increment form (built in shared memory
 // from the StepCoef table by fast_coef):
@@ -100,20 +107,24 @@ struct FastState {
 // G + a, which nearly cancel
 PF_FF_FN float rest_of(ff G, float a) { return f_add(f_add(G.h, a), G.l); }
 
-// dl = lo + d unless d is too large beside the state for an FP32 solution
+// every component of d at most t of y's (false if one is not finite)
+PF_FF_FN bool within(float t, float y1, float y2, float y3, float d1, float d2, float d3) {
+  return fabsf(d1) <= t * fabsf(y1) && fabsf(d2) <= t * fabsf(y2) && fabsf(d3) <= t * fabsf(y3);
+}
+
+// dl = lo + d; whether d is small enough beside the state for an FP32 solution
 PF_FF_FN bool rest_serves(const FastState& st, float y1, float y2, float y3, float d1, float d2, float d3,
                           ff (&dl)[3]) {
   dl[0] = two_sum(st.lo[0], d1);
   dl[1] = two_sum(st.lo[1], d2);
   dl[2] = two_sum(st.lo[2], d3);
-  return fabsf(d1) + fabsf(d2) + fabsf(d3) <= kFastRest * (fabsf(y1) + fabsf(y2) + fabsf(y3));
+  return within(kFastRest, y1, y2, y3, d1, d2, d3);
 }
 
 // ---------------------------------------------------------------- Robertson
 struct RobertsonFast {
   static constexpr int D = 3;
-  // f is quadratic: within rounding of the K-th iterate also at five substeps an interval
-  static constexpr float kSettled = 0x1.0p-12f;
+  static constexpr float kSettled = 1.0f;  // f is quadratic
   struct Fk {
     ff k1, k2, k3;          // theta
   };
@@ -198,10 +209,10 @@ struct RobertsonFast {
   }
 
   // the last iteration's correction.  fy, dfy: f at the corrected point (double
-  // part and ff part), if wanted
+  // part and ff part), if wanted.  False if the rest is above `settled` of the state.
   template <bool NEEDF, class Th>
-  PF_FF_FN static void last(const Th& T, const Fk& fk, const Gk& k, const FastCoef& c, const FastState& st,
-                            ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
+  PF_FF_FN static bool last(const Th& T, const Fk& fk, const Gk& k, const FastCoef& c, const FastState& st,
+                            float settled, ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
     const double y1 = st.y[0], y2 = st.y[1], y3 = st.y[2];
     const double q64 = T.k3 * y2;
     const double s64 = fma(T.k1, y1, -(q64 * y3));  // k1 y1 - k3 y2 y3 = -f1
@@ -217,7 +228,10 @@ struct RobertsonFast {
     float d1, d2, d3;
     solve32(k, q, p, w, rest_of(G1, f_add(st.lo[0], v)), rest_of(G2, f_add(f_sub(st.lo[1], v), wl)),
             rest_of(G3, f_sub(st.lo[2], wl)), d1, d2, d3);
-    if (!rest_serves(st, e1, e2f, e3, d1, d2, d3, dl)) solve(k, ff_from(y2), ff_from(y3), G1, G2, G3, dl);
+    if (!rest_serves(st, e1, e2f, e3, d1, d2, d3, dl)) {
+      if (!within(settled, e1, e2f, e3, d1, d2, d3)) return false;
+      solve(k, ff_from(y2), ff_from(y3), G1, G2, G3, dl);
+    }
     if (NEEDF) {
       const ff f2 = ff_from(y2), f3 = ff_from(y3);
       // f is quadratic: f(y + d) = f(y) + J d + Q(d, d), in ff beside FP64 f(y)
@@ -232,6 +246,7 @@ struct RobertsonFast {
       dfy[1] = ff_sub(ds, dc);
       dfy[2] = dc;
     }
+    return true;
   }
 };
 
@@ -241,9 +256,8 @@ struct RobertsonFast {
 // FP64 FMA, so no FP64 reciprocal is needed.
 struct MichaelisFast {
   static constexpr int D = 3;
-  // Iterates that jump past the pole x = -k do not settle (a tenth of the prior, in the
-  // first interval).  Over 300 particles of it the K-th iterate was up to 8e-9 off
-  // where corrections to 2^-4 were taken, 5e-13 to 2^-16, within FP64's rounding here.
+  // Iterates that jump past the pole x = -k do not settle (a fifth of the prior, in the
+  // first interval).
   static constexpr float kSettled = 0x1.0p-20f;
   struct Fk {
     double vk1, vk2, vd, vc;      // V1 k1, V2 k2, V1 - V2, V2 + lambda c0
@@ -338,8 +352,8 @@ struct MichaelisFast {
   }
 
   template <bool NEEDF, class Th>
-  PF_FF_FN static void last(const Th& T, const Fk& k, const Gk& gk, const FastCoef& c, const FastState& st,
-                            ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
+  PF_FF_FN static bool last(const Th& T, const Fk& k, const Gk& gk, const FastCoef& c, const FastState& st,
+                            float settled, ff (&dl)[3], double (&fy)[3], ff (&dfy)[3]) {
     const double s1 = st.y[0] + T.k1, s2 = st.y[1] + T.k2;
     const ff e1 = ff_from(s1), e2 = ff_from(s2);
     const ff r1 = ff_rcp(e1), r2 = ff_rcp(e2);
@@ -360,8 +374,11 @@ struct MichaelisFast {
     float d1, d2, d3;
     solve32(gk, ga, gb, rest_of(G1, f_add(st.lo[0], al)), rest_of(G2, f_sub(f_add(st.lo[1], bl), al)),
             rest_of(G3, f_sub(f_fma(gk.gl.h, st.lo[2], st.lo[2]), bl)), d1, d2, d3);
-    const bool rest = rest_serves(st, f_from(st.y[0]), f_from(st.y[1]), f_from(st.y[2]), d1, d2, d3, dl);
-    if (!rest) solve(gk, c, ff_add(du1, u1), r1, ff_add(du2, u2), r2, G1, G2, G3, dl);
+    const float y1 = f_from(st.y[0]), y2 = f_from(st.y[1]), y3 = f_from(st.y[2]);
+    if (!rest_serves(st, y1, y2, y3, d1, d2, d3, dl)) {
+      if (!within(settled, y1, y2, y3, d1, d2, d3)) return false;
+      solve(gk, c, ff_add(du1, u1), r1, ff_add(du2, u2), r2, G1, G2, G3, dl);
+    }
     if (NEEDF) {
       const ff t1 = ff_add(du1, u1), t2 = ff_add(du2, u2);
       // u(s + d) = u - u d/(s + d)
@@ -371,6 +388,7 @@ struct MichaelisFast {
       dfy[1] = ff_sub(v2, v1);
       dfy[2] = ff_neg(ff_add(v2, ff{0.5f * dl[2].h, 0.5f * dl[2].l}));
     }
+    return true;
   }
 };
 
@@ -400,17 +418,23 @@ struct FastCarry {
   ff fa[3], fb[3], fc[3], E[3];
 };
 
-// One substep.  FAM: 0 BDF2, 1 BDF3, 2 Adams-Moulton.  Returns false, with w
-// untouched, if the result is not to be trusted.
-template <class MF, int FAM, bool ERR, class Th>
-PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& c, int K, FastCarry& w) {
+// One substep.  FAM: 0 BDF2, 1 BDF3, 2 Adams-Moulton.  WIDE: every early iteration in
+// ff, from a start in ff, and the last at the (K-1)-th iterate to FP64 rounding instead
+// of a float's.
+//  kStepSettled   done, the rest below kFastSettled
+//  kStepWide      (WIDE) done, the rest above it
+//  kStepUnsettled (not WIDE) w untouched, to be taken again with WIDE
+//  kStepFar       w untouched, left to FP64
+enum { kStepSettled, kStepWide, kStepUnsettled, kStepFar };
+template <class MF, int FAM, bool ERR, bool WIDE, class Th>
+PF_FF_FN int fast_iterate(const Th& T, const typename MF::Fk& fk, const FastCoef& c, int K, FastCarry& w) {
   const typename MF::Gk gk = fast_scaled(T, fk, c);
   ff P[3], Dv[3], xf[3];
   FastState st;
   for (int i = 0; i < 3; ++i) {
     xf[i] = ff_add_raw(ff_from(w.x[i]), w.cx[i]);
-    if (!ERR && FAM != 2) {
-      // a start for the iterations only: a float does
+    if (!ERR && FAM != 2 && !WIDE) {
+      // a start for the iterations only: a float does, as an early FP32 solve does
       float p = f_fma(c.pb.h, w.fb[i].h, f_fma(c.pa.h, w.fa[i].h, f_mul(c.ep, xf[i].h)));
       if (FAM == 1) p = f_fma(c.pc.h, w.fc[i].h, p);
       Dv[i] = ff{p, 0.0f};
@@ -429,12 +453,12 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
       if (FAM != 0) R[i] = ff_fma(c.frb, w.fb[i], R[i]);
     }
     for (int it = 0; it + 1 < K; ++it) {
-      if (FAM != 2 && it + 2 < K) MF::first(fk, gk, c, xf, R, Dv);
-      else if (FAM == 2 && (it + 2 < K || K == 2)) MF::template early<true>(fk, gk, c, xf, R, Dv);
+      if (WIDE || (FAM == 2 && (it + 2 < K || K == 2))) MF::template early<true>(fk, gk, c, xf, R, Dv);
+      else if (it + 2 < K) MF::first(fk, gk, c, xf, R, Dv);
       else MF::template early<false>(fk, gk, c, xf, R, Dv);
     }
   }
-  float hh[3];
+  float hh[3], lw[3];  // lw: D's low float where the point has it (WIDE)
   for (int i = 0; i < 3; ++i) {
     // the point x + hh, hh the float nearest D + cx: from x_n it is hh - cx
     const ff s = ff_add(Dv[i], w.cx[i]);
@@ -450,24 +474,31 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
     if (FAM == 1) r = ff_fma(c.frb, w.rb[i], r);
     if (FAM != 2) r.l = f_fma(-c.er, xf[i].h, r.l);
     st.cor[i] = ff_sub_raw(r, w.cx[i]);
+    if (WIDE) {
+      lw[i] = s.l;
+      st.lo[i] = 0.0f;
+      st.y[i] += d_from_f(s.l);
+      st.cor[i] = ff_add(st.cor[i], s.l);
+    }
   }
   ff dl[3], dfy[3];
   double fy[3];
-  MF::template last<FAM != 0>(T, fk, gk, c, st, dl, fy, dfy);
-  // Every value finite and the last correction small beside the state.  The early
-  // solves leave the (K-1)-th iterate 2^-22 of its own step off, which the last
-  // iteration contracts by its distance from the solution, about |d|.
-  const float my = fabsf(f_from(st.y[0])) + fabsf(f_from(st.y[1])) + fabsf(f_from(st.y[2]));
-  const float md = fabsf(dl[0].h) + fabsf(dl[1].h) + fabsf(dl[2].h);
-  if (!(md <= (K > 1 ? MF::kSettled : kFastSingle) * my && my < 0x1.0p60f)) return false;
+  // (a single iteration has no earlier one to be off by: the ff solve of its rest is good to
+  // 2^-46 of it)
+  const float limit = !WIDE ? kFastSettled : K == 1 ? 1.0f : MF::kSettled;
+  if (!MF::template last<FAM != 0>(T, fk, gk, c, st, limit, dl, fy, dfy)) return WIDE ? kStepFar : kStepUnsettled;
+  // values still in the floats' range (and finite)
+  if (!(fabsf(f_from(st.y[0])) + fabsf(f_from(st.y[1])) + fabsf(f_from(st.y[2])) < 0x1.0p24f)) return kStepFar;
   if (ERR) {
     // and squares of the scaled estimates whose sum stays a float (640 of 2^116)
-    const float me = fabsf(P[0].h) + fabsf(P[1].h) + fabsf(P[2].h) + fabsf(hh[0]) + fabsf(hh[1]) + fabsf(hh[2]) + md;
-    if (!(fabsf(c.mus.h) * me < 0x1.0p58f)) return false;
+    float me = 0.0f;
+    for (int i = 0; i < 3; ++i) me = me + fabsf(P[i].h) + fabsf(hh[i]) + fabsf(dl[i].h);
+    if (!(fabsf(c.mus.h) * me < 0x1.0p58f)) return kStepFar;
   }
   for (int i = 0; i < 3; ++i) {
     // the increment from x_n to the new state
-    const ff rest = ff_sub(dl[i], w.cx[i]);
+    ff rest = ff_sub(dl[i], w.cx[i]);
+    if (WIDE) rest = ff_add(rest, lw[i]);
     const ff Dn = ff_add(rest, hh[i]);
     if (ERR) {
       const ff e = ff_mul(c.mus, ff_sub(Dn, P[i]));
@@ -502,7 +533,18 @@ PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& 
     w.x[i] = st.y[i];
     w.cx[i] = dl[i];
   }
-  return true;
+  if (!WIDE) return kStepSettled;
+  const float y1 = f_from(st.y[0]), y2 = f_from(st.y[1]), y3 = f_from(st.y[2]);
+  return within(kFastSettled, y1, y2, y3, dl[0].h, dl[1].h, dl[2].h) ? kStepSettled : kStepWide;
+}
+
+// One substep; false, with w untouched, if it is left to FP64.  (The kernels have the two
+// tries in loops of their own.)
+template <class MF, int FAM, bool ERR, class Th>
+PF_FF_FN bool fast_step(const Th& T, const typename MF::Fk& fk, const FastCoef& c, int K, FastCarry& w) {
+  int r = fast_iterate<MF, FAM, ERR, false>(T, fk, c, K, w);
+  if (r == kStepUnsettled) r = fast_iterate<MF, FAM, ERR, true>(T, fk, c, K, w);
+  return r == kStepSettled || r == kStepWide;
 }
 
 PF_FF_FN double ff_value(ff a) { return (double)a.h + (double)a.l; }

@@ -161,9 +161,34 @@ __device__ __forceinline__ int fast_run(const typename M::Th& T, const StepCoef*
 #pragma unroll
     for (int i = 0; i < 3; ++i) w.fc[i] = ff_from(fx[i]);
   }
+  // The lanes that got here go through the substeps together, so that fast_step's two
+  // forms are two loops (both in one loop: Robertson N = 131072 stages 266/327 us; loops
+  // that each lane leaves for itself: 536/1000, the warp in pieces).  After a substep that
+  // some lane has to take in the wide form, all take that form until all have settled.
+  unsigned lanes = __activemask();
+  auto serves = [&]() {
+    return s < S && fast_kind<F>(sc[s].kind) && fc[s].g.h >= kFastStepMin && fc[s].g.h <= kFastStepMax;
+  };
+  int r = kStepSettled;
 #pragma unroll 1
-  for (; s < S && fast_kind<F>(sc[s].kind) && fc[s].g.h >= kFastStepMin && fc[s].g.h <= kFastStepMax; ++s)
-    if (!fast_step<MF, FAM, ERR>(T, fk, fc[s], K, w)) break;
+  for (;;) {
+#pragma unroll 1
+    for (; serves(); ++s) {
+      r = fast_iterate<MF, FAM, ERR, false>(T, fk, fc[s], K, w);
+      if (__any_sync(lanes, r != kStepSettled)) break;
+    }
+    bool taken = r != kStepUnsettled;  // by this lane, the substep that ended the loop
+#pragma unroll 1
+    while (serves()) {
+      if (!taken) r = fast_iterate<MF, FAM, ERR, true>(T, fk, fc[s], K, w);
+      taken = false;
+      lanes = __ballot_sync(lanes, r != kStepFar);
+      if (r == kStepFar) break;
+      ++s;
+      if (!__any_sync(lanes, r == kStepWide)) break;
+    }
+    if (r == kStepFar || !serves()) break;
+  }
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     fast_history<FAM>(w, i, x[i], h1[i], h2[i]);
