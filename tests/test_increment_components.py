@@ -74,6 +74,37 @@ def test_robertson_components(shim, S, K, intervals, err):
     assert taken >= 0.9 * total
 
 
+@pytest.mark.parametrize("lmm", [W.LMM_BDF2, W.LMM_AM1, W.LMM_AM3])
+def test_michaelis_components(shim, lmm):
+    """Intervals after the first over the prior: a component is rounded once a substep (half
+    an ulp, 2^-53 of it at most), at random, so over the particles its error's root mean
+    square is at most sqrt(S) 2^-53, twice that allowed for the values converted on the way."""
+    if np.finfo(np.longdouble).eps > 2.0 ** -62:
+        pytest.skip("no extended precision on this machine")
+    w = W.michaelis(T=6, lmm=lmm)
+    cfg, rng = oracle.make_config(w), np.random.default_rng(78)
+    errs = []
+    for _ in range(40):
+        th = np.ascontiguousarray(np.exp(rng.uniform(np.log(w.prior_lo), np.log(w.prior_hi))))
+        x = h1 = h2 = np.array(w.x0)
+        t, depth, hp1, hp2 = 0.0, 0, 0.0, 0.0
+        for k in range(4):
+            tab, S, dout = oracle.build_substeps(cfg, t, w.t_obs[k], depth, hp1, hp2)
+            rows = oracle.substep_dicts(tab, S)
+            ref = _extended("michaelis", th, rows, 4, x, h1, h2)
+            if k > 0:
+                h = rows[0]["h"]
+                f = [oracle.ode_f(w.ode, th, v, rows[0]["tn"] - j * h) for j, v in enumerate((x, h1, h2))]
+                s, E, tbl = np.concatenate([x, h1, h2, *f]), np.zeros(3), _rows(rows, w)
+                n = shim.shim_run(1, 2 if lmm > 10 else 0, 1, th.ctypes.data, tbl.ctypes.data, S, 4, s.ctypes.data, E.ctypes.data)
+                if n == S:
+                    errs.append(np.asarray((s[:3] - ref[0]) / np.abs(ref[0]), dtype=float))
+            x, h1, h2 = (np.asarray(v, dtype=np.float64) for v in ref[:3])
+            t, depth, hp2, hp1 = w.t_obs[k], dout, rows[-2]["h"], rows[-1]["h"]
+    assert len(errs) >= 100
+    assert np.all(np.sqrt(np.mean(np.square(errs), axis=0)) <= 2 * np.sqrt(S) * 2.0 ** -53)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("problem,lmm", [("robertson", W.LMM_BDF2), ("michaelis", W.LMM_BDF2), ("michaelis", W.LMM_AM3)])
 def test_single_iteration_on_the_device(problem, lmm):
