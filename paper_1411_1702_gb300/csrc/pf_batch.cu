@@ -229,7 +229,7 @@ struct pf_batch {
   int* clear_dev = nullptr;
   // tiles and graph of the last active set
   std::vector<char> tiles_active;
-  size_t tiles_smem = 0;
+  int tiles_S = 0;
   cudaGraphExec_t graph = nullptr;
   int64_t captures = 0, epochs = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -334,14 +334,14 @@ static cudaError_t upload_tiles(pf_batch* b) {
 // Enqueue the phases on b->stream.  With a concurrent shape, each per-model
 // group of a phase forks onto two branches (the model with the most tiles on
 // the main branch) and joins before the next phase.
-static cudaError_t launch_phases(pf_batch* b, size_t smem, const Shape& shape, bool with_moments) {
+static cudaError_t launch_phases(pf_batch* b, int S_max, const Shape& shape, bool with_moments) {
   const FilterDev* fds = b->fds_dev;
   const EpochParams* const* eps = b->eps_dev;
   const BatchTile* T = b->tiles_dev;
   cudaError_t e = cudaSuccess;
   auto run = [&](int phase, int ode, int lmm, const Range& r, cudaStream_t st) {
     if (e == cudaSuccess && r.cnt > 0)
-      e = launch_batch_phase(phase, ode, lmm, fds, eps, T + r.off, r.cnt, smem, 0, st);
+      e = launch_batch_phase(phase, ode, lmm, fds, eps, T + r.off, r.cnt, S_max, 0, st);
   };
   // the groups of a phase, the largest on the main branch and (concurrent
   // shape) the others on the side branch
@@ -373,12 +373,12 @@ static cudaError_t launch_phases(pf_batch* b, size_t smem, const Shape& shape, b
   return e;
 }
 
-static cudaError_t capture(pf_batch* b, size_t smem, const Shape& shape, bool with_moments,
+static cudaError_t capture(pf_batch* b, int S_max, const Shape& shape, bool with_moments,
                            cudaGraphExec_t* out) {
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  cudaError_t le = launch_phases(b, smem, shape, with_moments);
+  cudaError_t le = launch_phases(b, S_max, shape, with_moments);
   e = cudaStreamEndCapture(b->stream, &g);
   if (le != cudaSuccess) e = le;
   if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
@@ -388,14 +388,14 @@ static cudaError_t capture(pf_batch* b, size_t smem, const Shape& shape, bool wi
 
 // Time each launch shape on the pending epoch's phases up to stage 2 (they
 // leave the committed state untouched and are idempotent), keep the fastest.
-static cudaError_t run_autotune(pf_batch* b, const std::vector<char>& active, size_t smem) {
+static cudaError_t run_autotune(pf_batch* b, const std::vector<char>& active, int S_max) {
   double best = 1e300;
   int best_i = 0;
   for (int i = 0; i < 4; ++i) {
     build_tiles(b, active, kShapes[i].order);
     cudaError_t e = upload_tiles(b);
     cudaGraphExec_t gx = nullptr;
-    if (e == cudaSuccess) e = capture(b, smem, kShapes[i], false, &gx);
+    if (e == cudaSuccess) e = capture(b, S_max, kShapes[i], false, &gx);
     double t = 1e300;
     for (int rep = 0; e == cudaSuccess && rep < 2; ++rep) {
       e = cudaEventRecord(b->ev0, b->stream);
@@ -631,9 +631,8 @@ static pf_status batch_launch(pf_batch* b, const double* t, const double* const*
   PF_BCUDA(b, cudaMemcpyAsync(b->slots_dev, b->slots_pin, sizeof(int) * n_act,
                               cudaMemcpyHostToDevice, b->stream));
   // 2-3. tiles, then the graph (active set seen before) or direct launches
-  const size_t smem = step_table_bytes(S_max);
-  if (b->autotune && !b->tuned) PF_BCUDA(b, run_autotune(b, active, smem));
-  const bool same = b->tiles_active == active && b->tiles_smem == smem;
+  if (b->autotune && !b->tuned) PF_BCUDA(b, run_autotune(b, active, S_max));
+  const bool same = b->tiles_active == active && b->tiles_S == S_max;
   if (!same) {
     if (b->graph) {
       cudaGraphExecDestroy(b->graph);
@@ -642,9 +641,9 @@ static pf_status batch_launch(pf_batch* b, const double* t, const double* const*
     build_tiles(b, active, b->shape.order);
     PF_BCUDA(b, upload_tiles(b));
     b->tiles_active = active;
-    b->tiles_smem = smem;
+    b->tiles_S = S_max;
   } else if (!b->graph) {
-    cudaError_t ce = capture(b, smem, b->shape, true, &b->graph);
+    cudaError_t ce = capture(b, S_max, b->shape, true, &b->graph);
     if (ce != cudaSuccess) {
       b->graph = nullptr;
       return bfail(b, PF_ERR_CUDA, std::string("graph capture failed: ") + cudaGetErrorString(ce));
@@ -655,7 +654,7 @@ static pf_status batch_launch(pf_batch* b, const double* t, const double* const*
   if (b->graph) {
     PF_BCUDA(b, cudaGraphLaunch(b->graph, b->stream));
   } else {
-    PF_BCUDA(b, launch_phases(b, smem, b->shape, true));
+    PF_BCUDA(b, launch_phases(b, S_max, b->shape, true));
   }
   PF_BCUDA(b, cudaEventRecord(b->ev1, b->stream));
   b->fl_done_ms = 0.0;

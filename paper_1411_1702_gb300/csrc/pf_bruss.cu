@@ -641,7 +641,7 @@ int bruss_stage_blocks(int64_t N) { return (int)((N + kBrPerBlock - 1) / kBrPerB
 
 cudaError_t launch_bruss_stage(int stage, const FilterDev& fd, const EpochParams* ep, int S,
                                cudaStream_t st) {
-  const size_t smem = step_table_bytes(S);
+  const size_t smem = step_table_bytes(PF_ODE_BRUSSELATOR1D, fd.lmm, S);
   const unsigned grid = (unsigned)bruss_stage_blocks(fd.N);
   if (stage == 1) k_bstage<1><<<grid, kBrThreads, smem, st>>>(fd, ep);
   else k_bstage<2><<<grid, kBrThreads, smem, st>>>(fd, ep);

@@ -104,13 +104,19 @@ __device__ __forceinline__ FastCoef* fast_table(const StepCoef* sc, int S) {
   return reinterpret_cast<FastCoef*>(const_cast<StepCoef*>(sc) + S);
 }
 
-// Both substep tables of a block in its dynamic shared memory
-// (step_table_bytes(S)).  Ends with a barrier.
-__device__ __forceinline__ void load_step_tables(StepCoef* s_sc, const EpochParams* __restrict__ ep, int S) {
+// The substep table of a block in its dynamic shared memory, and the increment form's
+// where the filter takes it (step_table_bytes: 200 B a substep, else 104).  Ends with a
+// barrier.
+template <class M, int F>
+__device__ __forceinline__ void load_step_tables(const FilterDev& fd, StepCoef* s_sc,
+                                                 const EpochParams* __restrict__ ep, int S) {
   load_steps(s_sc, ep, S);
-  FastCoef* t = fast_table(s_sc, S);
-  for (int i = threadIdx.x; i < S; i += blockDim.x) t[i] = fast_coef(s_sc[i]);
-  __syncthreads();
+  if constexpr (kHasFast<M, F>) {
+    if (fd.lmm == PF_LMM_BDF1) return;  // (no substep of its kind)
+    FastCoef* t = fast_table(s_sc, S);
+    for (int i = threadIdx.x; i < S; i += blockDim.x) t[i] = fast_coef(s_sc[i]);
+    __syncthreads();
+  }
 }
 
 // Whether the increment form takes a substep of this kind.
@@ -786,7 +792,7 @@ __global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_stage1(const
   // the parameter block is written only by copies before the epoch's first
   // launch, so its substep table is staged before the wait
   StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_step_tables(s_sc, ep, ep->S);
+  load_step_tables<M, F>(fd, s_sc, ep, ep->S);
   pdl_wait();
   if (fd.ctrl->status != PF_OK) return;
   stage1_body<M, F>(fd, ep, blockIdx.x, gridDim.x, s_sc, s_red, &s_flag);
@@ -827,7 +833,7 @@ __global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_stage2(const
   __shared__ double s_red[32];
   __shared__ int s_flag;
   StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_step_tables(s_sc, ep, ep->S);
+  load_step_tables<M, F>(fd, s_sc, ep, ep->S);
   pdl_wait();
   if (fd.ctrl->status != PF_OK) return;
   stage2_body<M, F>(fd, ep, blockIdx.x, gridDim.x, s_sc, s_red, &s_flag);
@@ -1006,7 +1012,7 @@ __global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_batch_stage(
   if (fd.ctrl->status != PF_OK) return;
   const EpochParams* ep = eps[t.f];
   StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_step_tables(s_sc, ep, ep->S);
+  load_step_tables<M, F>(fd, s_sc, ep, ep->S);
   const int vg = (int)((fd.N + kSmallThreads - 1) / kSmallThreads);
   if (STAGE == 1) stage1_body<M, F>(fd, ep, t.vb, vg, s_sc, s_red, &s_flag);
   else stage2_body<M, F>(fd, ep, t.vb, vg, s_sc, s_red, &s_flag);
@@ -1151,7 +1157,7 @@ template <class M>
 static cudaError_t launch_epoch_t(const FilterDev& fd, const EpochParams* ep, int S,
                                   cudaStream_t st, cudaEvent_t* marks) {
   const int64_t N = fd.N;
-  const size_t smem = step_table_bytes(S);
+  const size_t smem = step_table_bytes(M::ODE, fd.lmm, S);
   StageKernel k1, k2;
   stage_kernels<M>(fd.lmm, k1, k2);
   const unsigned g_small = stage_grid(N, fd.sms);
@@ -1294,11 +1300,16 @@ cudaError_t touch(K* k) {
 
 // A kernel that stages the substep table in dynamic shared memory may need
 // more than the default 48 KB (PF_MAX_SUBSTEPS entries); loads it as well.
-size_t step_table_bytes(int S) { return (sizeof(StepCoef) + sizeof(FastCoef)) * (size_t)S; }
+size_t step_table_bytes(int ode, int lmm, int S) {
+  const bool fast = ode == PF_ODE_BRUSSELATOR1D ||
+                    ((ode == PF_ODE_ROBERTSON || ode == PF_ODE_MICHAELIS3) && lmm != PF_LMM_BDF1 &&
+                     lmm_family(lmm) != kFamAb);
+  return (sizeof(StepCoef) + (fast ? sizeof(FastCoef) : 0)) * (size_t)S;
+}
 
 cudaError_t allow_step_table(const void* k) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)step_table_bytes(kSMax));
+                              (int)step_table_bytes(PF_ODE_BRUSSELATOR1D, PF_LMM_BDF2, kSMax));
 }
 
 struct UploadBlob {
@@ -1498,7 +1509,7 @@ cudaError_t launch_stage(int stage, const FilterDev& fd, const EpochParams* ep, 
     default: return cudaErrorInvalidValue;
   }
   const unsigned g = stage_grid(fd.N, fd.sms);
-  (stage == 1 ? k1 : k2)<<<g, stage_threads(fd.N, fd.sms), step_table_bytes(S), st>>>(fd, ep);
+  (stage == 1 ? k1 : k2)<<<g, stage_threads(fd.N, fd.sms), step_table_bytes(fd.ode, fd.lmm, S), st>>>(fd, ep);
   return cudaGetLastError();
 }
 
@@ -1567,16 +1578,17 @@ cudaError_t launch_set_moments(const FilterDev& fd, cudaStream_t st) {
 // One batched phase over the device tile table tiles[0..ntiles).  Stage and
 // moment phases need tiles of one model only (ode); the other phases take any
 // mix.
-// smem is the step-table size of the largest interval among the filters.
+// S is the substeps of the largest interval among the filters.
 cudaError_t launch_batch_phase(int phase, int ode, int lmm, const FilterDev* fds,
                                const EpochParams* const* eps, const BatchTile* tiles, int ntiles,
-                               size_t smem, int is_init, cudaStream_t st) {
+                               int S, int is_init, cudaStream_t st) {
   if (ntiles <= 0) return cudaSuccess;
   switch (phase) {
     case kPhaseInit: k_batch_init<<<ntiles, kInitThreads, 0, st>>>(fds, tiles); break;
     case kPhaseStage1:
     case kPhaseStage2: {
       const int stage = phase == kPhaseStage1 ? 1 : 2;
+      const size_t smem = step_table_bytes(ode, lmm, S);
       if (ode == PF_ODE_BRUSSELATOR1D)
         return launch_batch_bruss_stage(stage, fds, eps, tiles, ntiles, smem, st);
       BatchStageKernel k1, k2;

@@ -32,7 +32,7 @@ int bruss_stage_blocks(int64_t N);
 // moments those of one model.
 cudaError_t launch_batch_phase(int phase, int ode, int lmm, const FilterDev* fds,
                                const EpochParams* const* eps, const BatchTile* tiles, int ntiles,
-                               size_t smem, int is_init, cudaStream_t st);
+                               int S, int is_init, cudaStream_t st);
 // Batched Brusselator stage (1 or 2) over its own tile table (pf_bruss.cu).
 cudaError_t launch_batch_bruss_stage(int stage, const FilterDev* fds, const EpochParams* const* eps,
                                      const BatchTile* tiles, int ntiles, size_t smem,
@@ -68,9 +68,9 @@ cudaError_t launch_rows(const FilterDev& fd, int cur, cudaStream_t st);
 // Load every kernel of the library on the current device now rather than at
 // its first launch (which may wait for the device to drain); once per device.
 cudaError_t preload_main_kernels();
-// Dynamic shared memory of the small problems' stage kernels: the substep table
-// and the increment form's (pf_fast.cuh).
-size_t step_table_bytes(int S);
+// Dynamic shared memory of a problem's stage kernels for an LMM (of its family): the
+// substep table, and the increment form's (pf_fast.cuh) where the kernels read it.
+size_t step_table_bytes(int ode, int lmm, int S);
 // Let kernel k stage a full substep table (PF_MAX_SUBSTEPS entries) in dynamic
 // shared memory; loads the kernel.
 cudaError_t allow_step_table(const void* k);
