@@ -96,6 +96,37 @@ PF_FF_FN FastCoef fast_coef(const C& c) {
   return f;
 }
 
+#ifdef __CUDACC__
+// A block's substep tables: the steps, and the increment form's coefficients where the
+// kernel takes that form.  The second is formed in shared memory; the steps are copied
+// there while both leave room for four blocks an SM, and read where they were uploaded
+// in longer intervals (their uses are few beside the form, or the L1 cache serves them).  With
+// both always in shared memory an SM held one block at 640 substeps: Robertson N = 16384
+// stages 2914/3264 us.
+struct StepTables {
+  const StepCoef* sc;
+  const FastCoef* fc;
+};
+constexpr int kSharedTableBytes = 54 * 1024;
+__host__ __device__ constexpr int shared_steps_max(bool fast) {
+  return kSharedTableBytes / (int)(sizeof(StepCoef) + (fast ? sizeof(FastCoef) : 0));
+}
+__host__ __device__ constexpr bool steps_shared(int S, bool fast) { return S <= shared_steps_max(fast); }
+
+// Ends with a barrier.
+__device__ __forceinline__ StepTables load_step_tables(double* s_dyn, const EpochParams* __restrict__ ep, int S,
+                                                       bool fast) {
+  const bool shared = steps_shared(S, fast);
+  StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
+  if (shared) load_steps(s_sc, ep, S);
+  FastCoef* t = reinterpret_cast<FastCoef*>(shared ? s_sc + S : s_sc);
+  if (fast)
+    for (int i = threadIdx.x; i < S; i += blockDim.x) t[i] = fast_coef(ep->sc[i]);
+  __syncthreads();
+  return StepTables{shared ? s_sc : ep->sc, t};
+}
+#endif
+
 // the point of the last iteration, x_n + hh, and D + R of its residual: the leading
 // part in double, the rest in ff
 struct FastState {

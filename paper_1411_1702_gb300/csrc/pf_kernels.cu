@@ -99,23 +99,18 @@ struct FastModel<Michaelis> {
 template <class M, int F>
 constexpr bool kHasFast = !std::is_same<typename FastModel<M>::type, void>::value && F != kFamAb;
 
-// The increment form's table, behind the S entries of the substep table.
-__device__ __forceinline__ FastCoef* fast_table(const StepCoef* sc, int S) {
-  return reinterpret_cast<FastCoef*>(const_cast<StepCoef*>(sc) + S);
-}
 
-// The substep table of a block in its dynamic shared memory, and the increment form's
-// where the filter takes it (step_table_bytes: 200 B a substep, else 104).  Ends with a
-// barrier.
-template <class M, int F>
-__device__ __forceinline__ void load_step_tables(const FilterDev& fd, StepCoef* s_sc,
-                                                 const EpochParams* __restrict__ ep, int S) {
-  load_steps(s_sc, ep, S);
+// body() with the block's substep tables (StepTables), after a barrier.
+template <class M, int F, class Body>
+__device__ __forceinline__ void with_step_tables(const FilterDev& fd, double* s_dyn,
+                                                 const EpochParams* __restrict__ ep, Body body) {
+  const int S = ep->S;
   if constexpr (kHasFast<M, F>) {
-    if (fd.lmm == PF_LMM_BDF1) return;  // (no substep of its kind)
-    FastCoef* t = fast_table(s_sc, S);
-    for (int i = threadIdx.x; i < S; i += blockDim.x) t[i] = fast_coef(s_sc[i]);
-    __syncthreads();
+    body(load_step_tables(s_dyn, ep, S, fd.lmm != PF_LMM_BDF1));  // (BDF1: no substep of the form's kind)
+  } else {
+    // a copy of the body each, so that the usual one's reads are known to be shared
+    if (steps_shared(S, false)) body(load_step_tables(s_dyn, ep, S, false));
+    else body(StepTables{ep->sc, nullptr});
   }
 }
 
@@ -129,12 +124,13 @@ __device__ __forceinline__ bool fast_kind(int kind) {
 // serves the particle; returns the first substep it has not done.  (f0, f1,
 // f2: the derivative history of the Adams methods, in and out.)
 template <class M, bool ERR, int F, int NF>
-__device__ __forceinline__ int fast_run(const typename M::Th& T, const StepCoef* sc, int s, int S, int K,
+__device__ __forceinline__ int fast_run(const typename M::Th& T, const StepTables& tables, int s, int S, int K,
                                         double (&x)[3], double (&h1)[3], double (&h2)[3], double (&E)[3],
                                         double (&f0)[NF], double (&f1)[NF], double (&f2)[NF]) {
+  const StepCoef* sc = tables.sc;
+  const FastCoef* fc = tables.fc;
   using MF = typename FastModel<M>::type;
   constexpr int FAM = F == kFamBdf12 ? 0 : F == kFamBdf3 ? 1 : 2;
-  const FastCoef* fc = fast_table(sc, S);
   // every state and parameter in the range in which the floats serve
   double big = 0.0;
 #pragma unroll
@@ -223,12 +219,13 @@ __device__ __forceinline__ int fast_run(const typename M::Th& T, const StepCoef*
 // stops where that form can take over (after a cold start's BDF1 steps), the
 // second finishes what it left (for most particles nothing).
 template <class M, bool ERR, int F>
-__device__ __forceinline__ void propagate(const typename M::Th& T, const StepCoef* sc, int S, int K,
+__device__ __forceinline__ void propagate(const typename M::Th& T, const StepTables& tables, int S, int K,
                                           const EpochParams* __restrict__ ep, double (&x)[M::D],
                                           double (&h1)[M::D], double (&h2)[M::D], double (&E)[M::D]) {
   constexpr int D = M::D;
   constexpr bool kAdams = F == kFamAm || F == kFamAb;
   constexpr bool kFast = kHasFast<M, F>;
+  const StepCoef* sc = tables.sc;
   double f0[kAdams ? D : 1], f1[kAdams ? D : 1], f2[kAdams ? D : 1];
   if constexpr (kAdams) {
     const int q0 = sc[0].kind % 10;
@@ -333,7 +330,7 @@ __device__ __forceinline__ void propagate(const typename M::Th& T, const StepCoe
       }
     }
     if constexpr (kFast) {
-      if (pass == 0) s = fast_run<M, ERR, F>(T, sc, s, S, K, x, h1, h2, E, f0, f1, f2);
+      if (pass == 0) s = fast_run<M, ERR, F>(T, tables, s, S, K, x, h1, h2, E, f0, f1, f2);
     }
   }
 }
@@ -382,7 +379,7 @@ __device__ __forceinline__ void init_body(const FilterDev& fd, int vb) {
 // ---------------------------------------------------------------- stage 1
 template <class M, int F>
 __device__ __forceinline__ void stage1_body(const FilterDev& fd, const EpochParams* __restrict__ ep,
-                                            int vb, int vg, const StepCoef* s_sc, double* s_red,
+                                            int vb, int vg, const StepTables& tables, double* s_red,
                                             int* s_flag) {
   constexpr int D = M::D, P = M::P;
   const Ctrl* ctrl = fd.ctrl;
@@ -404,7 +401,7 @@ __device__ __forceinline__ void stage1_body(const FilterDev& fd, const EpochPara
       h1[i] = E.h1[i * N + n];
       h2[i] = E.h2[i * N + n];
     }
-    propagate<M, false, F>(T, s_sc, S, fd.K, ep, x, h1, h2, Eunused);
+    propagate<M, false, F>(T, tables, S, fd.K, ep, x, h1, h2, Eunused);
     const double ll = loglik<D>(fd, ep, x);
     fd.ll1[n] = ll;
     lg = (E.lw[n] - ctrl->logW) + ll;
@@ -461,7 +458,7 @@ __device__ __forceinline__ void resample_body(const FilterDev& fd, const EpochPa
 // ---------------------------------------------------------------- stage 2
 template <class M, int F>
 __device__ __forceinline__ void stage2_body(const FilterDev& fd, const EpochParams* __restrict__ ep,
-                                            int vb, int vg, const StepCoef* s_sc, double* s_red,
+                                            int vb, int vg, const StepTables& tables, double* s_red,
                                             int* s_flag) {
   constexpr int D = M::D, P = M::P;
   const Ctrl* ctrl = fd.ctrl;
@@ -503,7 +500,7 @@ __device__ __forceinline__ void stage2_body(const FilterDev& fd, const EpochPara
       Eacc[i] = 0.0;
     }
     // 4b, 4d: repropagate, summing the squared Milne estimates
-    propagate<M, true, F>(T, s_sc, S, fd.K, ep, x, h1, h2, Eacc);
+    propagate<M, true, F>(T, tables, S, fd.K, ep, x, h1, h2, Eacc);
     // 4c, 4d: v ~ N(0, kappa diag(E)), added to x and to the stored history
 #pragma unroll
     for (int b = 0; b < (D + 1) / 2; ++b) {
@@ -791,11 +788,11 @@ __global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_stage1(const
   __shared__ int s_flag;
   // the parameter block is written only by copies before the epoch's first
   // launch, so its substep table is staged before the wait
-  StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_step_tables<M, F>(fd, s_sc, ep, ep->S);
-  pdl_wait();
-  if (fd.ctrl->status != PF_OK) return;
-  stage1_body<M, F>(fd, ep, blockIdx.x, gridDim.x, s_sc, s_red, &s_flag);
+  with_step_tables<M, F>(fd, s_dyn, ep, [&](const StepTables& tables) {
+    pdl_wait();
+    if (fd.ctrl->status != PF_OK) return;
+    stage1_body<M, F>(fd, ep, blockIdx.x, gridDim.x, tables, s_red, &s_flag);
+  });
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_tile(const __grid_constant__ FilterDev fd) {
@@ -832,11 +829,11 @@ __global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_stage2(const
   extern __shared__ double s_dyn[];
   __shared__ double s_red[32];
   __shared__ int s_flag;
-  StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_step_tables<M, F>(fd, s_sc, ep, ep->S);
-  pdl_wait();
-  if (fd.ctrl->status != PF_OK) return;
-  stage2_body<M, F>(fd, ep, blockIdx.x, gridDim.x, s_sc, s_red, &s_flag);
+  with_step_tables<M, F>(fd, s_dyn, ep, [&](const StepTables& tables) {
+    pdl_wait();
+    if (fd.ctrl->status != PF_OK) return;
+    stage2_body<M, F>(fd, ep, blockIdx.x, gridDim.x, tables, s_red, &s_flag);
+  });
 }
 
 template <int D, int P>
@@ -1011,11 +1008,11 @@ __global__ void __launch_bounds__(kSmallThreads, kStageBlocks<M>) k_batch_stage(
   const FilterDev& fd = *(fds + t.f);
   if (fd.ctrl->status != PF_OK) return;
   const EpochParams* ep = eps[t.f];
-  StepCoef* s_sc = reinterpret_cast<StepCoef*>(s_dyn);
-  load_step_tables<M, F>(fd, s_sc, ep, ep->S);
   const int vg = (int)((fd.N + kSmallThreads - 1) / kSmallThreads);
-  if (STAGE == 1) stage1_body<M, F>(fd, ep, t.vb, vg, s_sc, s_red, &s_flag);
-  else stage2_body<M, F>(fd, ep, t.vb, vg, s_sc, s_red, &s_flag);
+  with_step_tables<M, F>(fd, s_dyn, ep, [&](const StepTables& tables) {
+    if (STAGE == 1) stage1_body<M, F>(fd, ep, t.vb, vg, tables, s_red, &s_flag);
+    else stage2_body<M, F>(fd, ep, t.vb, vg, tables, s_red, &s_flag);
+  });
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_batch_scan_tile(const FilterDev* __restrict__ fds,
@@ -1300,16 +1297,23 @@ cudaError_t touch(K* k) {
 
 // A kernel that stages the substep table in dynamic shared memory may need
 // more than the default 48 KB (PF_MAX_SUBSTEPS entries); loads it as well.
+static bool has_fast(int ode, int lmm) {
+  return (ode == PF_ODE_ROBERTSON || ode == PF_ODE_MICHAELIS3) && lmm != PF_LMM_BDF1 && lmm_family(lmm) != kFamAb;
+}
 size_t step_table_bytes(int ode, int lmm, int S) {
-  const bool fast = ode == PF_ODE_BRUSSELATOR1D ||
-                    ((ode == PF_ODE_ROBERTSON || ode == PF_ODE_MICHAELIS3) && lmm != PF_LMM_BDF1 &&
-                     lmm_family(lmm) != kFamAb);
-  return (sizeof(StepCoef) + (fast ? sizeof(FastCoef) : 0)) * (size_t)S;
+  if (ode == PF_ODE_BRUSSELATOR1D) return (size_t)S * (sizeof(StepCoef) + sizeof(FastCoef));
+  const bool fast = has_fast(ode, lmm);
+  return (size_t)S * ((steps_shared(S, fast) ? sizeof(StepCoef) : 0) + (fast ? sizeof(FastCoef) : 0));
+}
+size_t step_table_room(int ode, int lmm, int S) {
+  const int most = shared_steps_max(has_fast(ode, lmm));
+  const size_t a = step_table_bytes(ode, lmm, S), b = step_table_bytes(ode, lmm, S < most ? S : most);
+  return a > b ? a : b;
 }
 
 cudaError_t allow_step_table(const void* k) {
   return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)step_table_bytes(PF_ODE_BRUSSELATOR1D, PF_LMM_BDF2, kSMax));
+                              (int)step_table_room(PF_ODE_BRUSSELATOR1D, PF_LMM_BDF2, kSMax));
 }
 
 struct UploadBlob {
@@ -1588,7 +1592,7 @@ cudaError_t launch_batch_phase(int phase, int ode, int lmm, const FilterDev* fds
     case kPhaseStage1:
     case kPhaseStage2: {
       const int stage = phase == kPhaseStage1 ? 1 : 2;
-      const size_t smem = step_table_bytes(ode, lmm, S);
+      const size_t smem = step_table_room(ode, lmm, S);  // (members with fewer substeps too)
       if (ode == PF_ODE_BRUSSELATOR1D)
         return launch_batch_bruss_stage(stage, fds, eps, tiles, ntiles, smem, st);
       BatchStageKernel k1, k2;

@@ -71,6 +71,8 @@ cudaError_t preload_main_kernels();
 // Dynamic shared memory of a problem's stage kernels for an LMM (of its family): the
 // substep table, and the increment form's (pf_fast.cuh) where the kernels read it.
 size_t step_table_bytes(int ode, int lmm, int S);
+// the most of it for any interval of up to S substeps
+size_t step_table_room(int ode, int lmm, int S);
 // Let kernel k stage a full substep table (PF_MAX_SUBSTEPS entries) in dynamic
 // shared memory; loads the kernel.
 cudaError_t allow_step_table(const void* k);
