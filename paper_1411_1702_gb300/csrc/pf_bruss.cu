@@ -278,6 +278,12 @@ __device__ __noinline__ void br_step_fp64(const BrTheta& T, const StepCoef& c, i
                                           bool b64, bool mine) {
   double D0[4], P[4], R[4], xn[4], h1[4];
   double f[4];
+  // (a correction of 2^-13 of the state leaves a carry of 2^-38)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    w.x[k] += (double)w.cx[k];
+    w.a[k] += (double)w.ca[k];
+  }
   br_f(T, w.x, g, f);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
