@@ -12,7 +12,7 @@ from parity_util import begin_epoch
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("K,S", [(2, 5), (2, 20)])
+@pytest.mark.parametrize("K,S", [(2, 5), (2, 20), (1, 5), (1, 20)])
 def test_kth_iterate(K, S):
     B.build()
     oracle.build()
