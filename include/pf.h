@@ -267,7 +267,8 @@ pf_status pf_reset(pf_filter* f);
 /* ---- checkpoint and inspection ------------------------------------------
  * Copy the committed ensemble to or from host memory: x, h1, h2 (N*d each:
  * x_n and the two previous LMM substep states), phi (N*p) and the normalised
- * log weights logw (N).  Any pointer may be NULL (not copied).  Setting the
+ * log weights logw (N).  Any pointer may be NULL (not copied).  If reading
+ * fails, what was to be filled is unspecified.  Setting the
  * ensemble does not recompute the moments; use pf_set_moments. */
 pf_status pf_get_ensemble(const pf_filter* f, double* x, double* h1, double* h2, double* phi,
                           double* logw);

@@ -25,7 +25,7 @@
 // What FP64 is needed for (an FP64 instruction costs the time of 64 FP32 ones on
 // GB300, a 32x32-bit integer multiply-add into 64 bits that of five or six):
 //  - the mode steps X_{n+1} = W (X_n + kappa X_{n-1}), W = rho1/(1 - gamma lambda)
-//    complex, kappa = rho2/rho1: 6 FP64 instructions a mode.  The substeps of a
+//    complex, kappa = rho2/rho1: 8 FP64 instructions a mode.  The substeps of a
 //    uniform grid have gammas that differ in their last bits; W is formed for the
 //    first and the others' difference applied to first order in FP32.
 //  - Milne's estimate mu (X_{n+1} - X_p) while it is not small beside the state:

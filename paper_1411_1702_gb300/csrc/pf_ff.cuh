@@ -13,7 +13,8 @@
 // on the integer pipe: the conversion instructions between the two formats run
 // at the FP64 rate (two lanes a clock, measured).
 //
-// A host build (tests) gives the same bits.
+// A host build (tests) gives the same bits but for the reciprocal's last one and the sign
+// of a NaN.
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -158,7 +159,8 @@ PF_FF_FN float f_from(double a) {
   if (v - 0x00100000u >= 0x0fe00000u) b = (int32_t)v < 0x00100000 ? 0u : 0x7f800000u;
   return f_from_bits(b | (hi & 0x80000000u));
 }
-// exact for finite f; below the least normal float it gives 0
+// exact for finite f; below the least normal float it gives 0 (an infinity or a NaN
+// would become a number of 2^128: no caller passes one on)
 PF_FF_FN double d_from_f(float f) {
   const uint32_t b = f_bits(f), m = b & 0x7fffffffu;
   const bool none = m < 0x00800000u;

@@ -44,8 +44,9 @@ constexpr int kInitThreads = 256;
 // More warps hide the waits on FP64 results.  Unbounded, Robertson's stage 2 took 159
 // registers and M1's 188, whose 10 resident warps an SM left M1's 10.3 warps an SM at N
 // = 50000 with a second wave: M1 stage 2 0.129 -> 0.088 ms, AM3's 0.152 -> 0.101;
-// Robertson stage 2 0.373 -> 0.347 ms at N = 131072.  168 for Robertson slowed its
-// stage 1 by 17 % and 128 for M1 both of its stages by 4 %.
+// Robertson stage 2 0.373 -> 0.347 ms at N = 131072.  168 for Robertson slows every
+// family (N = 131072: BDF2 241/306 -> 298/363 us, BDF3 330/427 -> 399/508, AM3 360/447 ->
+// 391/518, though at 128 AM3's stage 2 spills 1 KB), 128 for M1 both of its stages by 4 %.
 template <class M>
 constexpr int kStageBlocks = M::ODE == PF_ODE_MICHAELIS3 ? 3 : 4;
 
@@ -166,7 +167,9 @@ __device__ __forceinline__ int fast_run(const typename M::Th& T, const StepTable
   // The lanes that got here go through the substeps together, so that fast_step's two
   // forms are two loops (both in one loop: Robertson N = 131072 stages 266/327 us; loops
   // that each lane leaves for itself: 536/1000, the warp in pieces).  After a substep that
-  // some lane has to take in the wide form, all take that form until all have settled.
+  // some lane has to take in the wide form, all take that form until all have settled, so
+  // a particle's last bits depend on its 32: slots 32 i to 32 i + 31, the same alone, in
+  // a batch and in a shard.
   unsigned lanes = __activemask();
   auto serves = [&]() {
     return s < S && fast_kind<F>(sc[s].kind) && fc[s].g.h >= kFastStepMin && fc[s].g.h <= kFastStepMax;

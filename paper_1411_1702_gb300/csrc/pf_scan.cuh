@@ -88,11 +88,11 @@ __device__ __forceinline__ int32_t systematic_index(const V& c, int64_t N, int64
 // exact and associative, so c is a deterministic function of the log weights
 // for a given N.
 //
-// The exponentials are the scan's cost and FP64 issue is scarce, so the tile
-// length follows N and the device's SM count: of 1 to kScanItemsMax values a
+// The tile length follows N and the device's SM count: of 1 to kScanItemsMax values a
 // thread, the one whose busiest SM has the least to do -- ceil(tiles / sms)
-// tiles of (items + 0.3) units, the 0.3 standing for a thread's share of the
-// block scan -- among those that keep the tile count at most
+// tiles of (items + 0.3) units, a unit an exponential and its sum, the 0.3 standing for
+// a thread's share of the block scan (a ratio measured with FP64 exponentials; the
+// fixed-point ones cost less) -- among those that keep the tile count at most
 // max(kScanTilesPerSm * sms, ceil(N / (kScanThreads * kScanItemsMax))); ties
 // go to more values a thread.
 __host__ __device__ constexpr int scan_items(int64_t N, int sms) {
