@@ -28,7 +28,7 @@ def _scaled(n, N, T, k):
 
 
 @pytest.mark.parametrize("n,N,T", [(20, 9, 2), (40, 3, 1)])
-@pytest.mark.parametrize("k", [34, 45, 70, -30, -60])
+@pytest.mark.parametrize("k", [34, 45, 70, 300, -30, -60, -300])
 def test_scaled_epochs(pf, n, N, T, k):
     runs = []
     for w in (_scaled(n, N, T, 0), _scaled(n, N, T, k)):
