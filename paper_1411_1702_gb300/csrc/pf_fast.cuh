@@ -52,14 +52,15 @@ constexpr float kFastStepMin = 0x1.0p-60f, kFastStepMax = 0x1.0p40f;
 //    solved for in ff (0.3 % of Robertson's substeps over its prior at S = 50, K = 2).
 //  - The point is off the (K-1)-th iterate by D's rounding to a float, and that by the
 //    early FP32 solves' 2^-22 of their step; the last iteration leaves both times the
-//    rest.  Above 2^-17 the substep is taken with all of that in ff and FP64 (WIDE): a few
+//    rest.  Above 2^-15 the substep is taken with all of that in ff and FP64 (WIDE): a few
 //    at the start of intervals whose parameters have just moved (stage 2: up to half a
 //    dozen of 50), and every one of K = 1.  The models' kSettled is what the rest may be
 //    then; a substep above it goes to FP64.  Over Robertson's prior, parameters moved by a
-//    fifth, y2 and y3 are within 5e-16 (S = 50, K = 2; FP64 path 3e-15) and 7e-15 (S = 2; 2e-10);
-//    limits of 2^-19 to 2^-26 give the same at S = 50.  With limits on the norm and no second
-//    form it was 1e-13 and 2e-10, and up to 6e-9 for K = 1.
-constexpr float kFastRest = 0x1.0p-32f, kFastSettled = 0x1.0p-17f;
+//    fifth, y2 and y3 are within 5e-16 (S = 50, K = 2; FP64 path 3e-15), 2e-15 (S = 10; 8e-12),
+//    4e-14 (S = 5; 1e-7).  2^-17 to 2^-26 give the same at S = 50 and cost more (0.588 ms a
+//    Robertson epoch at 2^-17, 0.578 here, 0.572 with no second form); with limits on the norm
+//    and no second form it was 1e-13, 3e-12 and 2e-7, and up to 6e-9 for K = 1.
+constexpr float kFastRest = 0x1.0p-32f, kFastSettled = 0x1.0p-15f;
 
 // One substep's coefficients for the increment form (built in shared memory
 // from the StepCoef table by fast_coef):
