@@ -160,15 +160,15 @@ STAGE2_KERNEL["michaelis"] = "k_stage2<Michaelis, 0>"
 # DRAM bytes (read + write) of one stage-2 launch from an ncu capture of the
 # same command on a GB300 (profiles/ names each capture); None where no capture
 # of the kernel as it stands exists.
-STAGE2_TRAFFIC = {"robertson": 11579136 + 0,
-                  "brusselator": 96326656 + 59988480,
-                  "advdiff20": 3375104 + 20635904,
-                  "advdiff40": 179305472 + 197228032,
-                  "michaelisBDF2": 4390144 + 0}
+STAGE2_TRAFFIC = {"robertson": 11582720 + 0,
+                  "brusselator": 96534528 + 60008448,
+                  "advdiff20": 3412480 + 18903040,
+                  "advdiff40": 179368960 + 189291264,
+                  "michaelisBDF2": 4393216 + 0}
 # FP64 warp instructions of the same launches (sm__inst_executed_pipe_fp64.sum):
 # each holds its SM sub-partition's FP64 pipe for 64 cycles.
-STAGE2_FP64_WARPS = {"robertson": 4012033, "brusselator": 35987457, "advdiff20": 13380309,
-                     "advdiff40": 52583037, "michaelisBDF2": 758056}
+STAGE2_FP64_WARPS = {"robertson": 4012033, "brusselator": 35987457, "advdiff20": 13442809,
+                     "advdiff40": 52828037, "michaelisBDF2": 711166}
 # The paper's own number for the same workload, where it has one: Table 3's
 # 2D advection-diffusion runs (BDF2, h = 0.1, N = 5000, 30 unit intervals,
 # 8 MATLAB workers on an i7-3820), converted to particle-LMM-steps/s at 600

@@ -575,8 +575,9 @@ __device__ __forceinline__ ff bits_ff(double a) { return ff{f_from_bits(d_hi(a))
 // n = 20, N = 5000 stage 2 0.95 against 1.70 ms, n = 40, N = 1000 1.11 against
 // 1.40 ms, the state's transform then still in integers).
 // Measured (GB300), against FP64 transforms and mode steps throughout: n = 20,
-// N = 5000 stage 1 0.82 -> 0.41 ms, stage 2 2.26 -> 0.96 ms; n = 40, N = 1000 0.93 ->
-// 0.44, 2.89 -> 1.18 ms; the FP64 pipe is 85 and 68 % busy at n = 20, 77 and 52 % at 40.
+// N = 5000 stage 1 0.82 -> 0.41 ms, stage 2 2.26 -> 0.97 ms (1.05 with a cold cache); n = 40,
+// N = 1000 0.93 -> 0.43, 2.89 -> 1.14 ms; the FP64 pipe is 85 and 68 % busy at n = 20, 79 and
+// 51 % at 40.
 template <int STAGE, int U, int PB, int MAXT>
 __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 1 : MAXT == 416 || U == 2 ? 2 : 3) k_adstage(const __grid_constant__ FilterDev fd,
                                                                    const EpochParams* __restrict__ ep) {

@@ -17,7 +17,7 @@
 //   - the last evaluates G in FP64 at the point y = x_n + (leading float of D).
 //     Its correction is D's low float, known, plus a rest of about 2^-50 |y| that an
 //     FP32 solution serves; what FP32 made of the point does not matter, since G
-//     is evaluated at the point itself.  (A rest above 2^-34 |y| solves in ff.)
+//     is evaluated at the point itself.  (A larger rest, kFastRest below, solves in ff.)
 // The state stays the double of the last iteration's point plus that iteration's
 // correction in ff, so a substep rounds it once, and Milne's estimate comes from
 // D - P without the cancellation of y - x_p.  The result is the K-th Newton
@@ -26,12 +26,12 @@
 // exponent outside the floats') is left to the FP64 path by fast_run's caller.
 //
 // A Robertson BDF2 substep with error sums takes 15 FP64 instructions instead
-// of 89, an M1 one 19 instead of 186.  Measured (GB300, device time):
-// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.231 ms, stage 2 1.08 -> 0.290 ms;
-// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.065 and 0.23 -> 0.075 ms (the exponentials and
+// of 89, an M1 one 16 instead of 186.  Measured (GB300, device time):
+// Robertson, N = 131072, S = 50: stage 1 0.93 -> 0.237 ms, stage 2 1.08 -> 0.300 ms;
+// M1 BDF2, N = 50000, S = 10: 0.16 -> 0.062 and 0.23 -> 0.076 ms (the exponentials and
 // roots of pf_math.cuh and the register bounds included).  Accuracy over an interval,
 // against quadruple precision on 200 particles of the prior, 2-norm of the state:
-// Robertson 3e-17 (plain FP64 9e-16), M1 6e-17 (4e-16).
+// Robertson 3e-17 (plain FP64 9e-16), M1 6e-17 (4e-16); by component at kFastRest.
 #pragma once
 #include "pf_ff.cuh"
 
